@@ -139,11 +139,14 @@ int ensure_workspace(kl_solver* h, int k) {
     if (e != cudaSuccess) return cuda_fail(h, e, "workspace sync");
     clear_graphs(h);
     for (int i = 0; i < 3; ++i) {
+        if (h->ws[i]) h->dev_bytes -= std::max(h->S, h->T) * int64_t(h->k_cap) * int64_t(sizeof(double));
         dfree(h->ws[i]);
         h->ws[i] = nullptr;
     }
+    if (h->pair_scratch) h->dev_bytes -= h->pair_scratch_len * int64_t(sizeof(double));
     dfree(h->pair_scratch);
     h->pair_scratch = nullptr;
+    h->k_cap = 0;
     const int64_t big = std::max(h->S, h->T) * int64_t(k);
     for (int i = 0; i < 3; ++i)
         if ((e = dalloc(h, &h->ws[i], big)) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
