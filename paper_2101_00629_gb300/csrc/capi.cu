@@ -116,6 +116,19 @@ void domain_centre(const kl_params& p, double c[3]) {
     }
 }
 
+// Length of the domain along each parametric direction (mean arc for the
+// annuli, the cube's edges for its projective image).
+void domain_extent(const kl_params& p, double* e) {
+    const bool half = p.geometry == KL_GEOM_HALF_ANNULUS;
+    if (half || p.geometry == KL_GEOM_QUARTER_ANNULUS) {
+        e[0] = (half ? 1.0 : 0.5) * 3.14159265358979 * 0.5 * (p.geo[0] + p.geo[1]);
+        e[1] = p.geo[1] - p.geo[0];
+        e[2] = p.geo[2];
+    } else {
+        e[0] = e[1] = e[2] = 1.0;
+    }
+}
+
 template <class T>
 cudaError_t dalloc(kl_solver* h, T** p, int64_t count) {
     *p = nullptr;
@@ -264,6 +277,9 @@ static int pairwise(kl_solver* h, int precision, const double* U, double* W, int
         a.tx32 = h->tx32; a.ty32 = h->ty32; a.tz32 = h->tz32;
         a.sx32 = h->sx32; a.sy32 = h->sy32; a.sz32 = h->sz32;
         a.T = h->T; a.S = h->S;
+        double extent[3];
+        domain_extent(h->prm, extent);
+        for (int d = 0; d < 3; ++d) a.sn[d] = h->Ns1[d], a.sh[d] = extent[d] / h->Ns1[d];
         a.X = U; a.ldx = h->S; a.Y = W; a.ldy = h->T; a.k = k;
         a.post = post; a.ks = ks;
         a.scratch = h->pair_scratch; a.splits = h->pair_splits;

@@ -43,10 +43,29 @@ __host__ __device__ inline uint32_t mulhi32(uint32_t a, uint32_t b) {
 #endif
 }
 __host__ __device__ inline uint64_t mulwide(uint32_t a, uint32_t b) { return uint64_t(a) * b; }
+// a b + c, one multiply-add each
+__host__ __device__ inline uint64_t madwide(uint32_t a, uint32_t b, uint64_t c) {
+#ifdef __CUDA_ARCH__
+    uint64_t d;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+#else
+    return uint64_t(a) * b + c;
+#endif
+}
+__host__ __device__ inline int64_t madwide_s(int32_t a, int32_t b, int64_t c) {
+#ifdef __CUDA_ARCH__
+    int64_t d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+#else
+    return int64_t(a) * b + c;
+#endif
+}
 // high half of a 64 x 64-bit product, up to two units low
 __host__ __device__ inline uint64_t mulhi64(uint64_t a, uint64_t b) {
     const uint32_t ah = uint32_t(a >> 32), bh = uint32_t(b >> 32);
-    return mulwide(ah, bh) + mulhi32(ah, uint32_t(b)) + mulhi32(uint32_t(a), bh);
+    return madwide(ah, bh, mulhi32(ah, uint32_t(b))) + mulhi32(uint32_t(a), bh);
 }
 
 // 2^-(i / 2048) in units of 2^-63, i = 0..2047: products of the eleven
@@ -87,8 +106,8 @@ __host__ __device__ __forceinline__ uint64_t exp2_neg(uint64_t t, const uint64_t
     const uint32_t v = 0xf5fdefcbu - (mulhi32(r, 0xe34e6d62u) >> 13);  // c2 - c3 r, 2^-34
     const uint32_t w = mulhi32(r, v);                                  // 2^-45
     // c1 r - w r, 2^-75
-    uint64_t p = mulwide(r, 0xb17217f7u) + mulhi32(r, 0xd180aefeu);
-    p += rl * (Q == 55 ? 0xb1721u : 0x2c5c86u);
+    uint64_t p = madwide(r, 0xb17217f7u, mulhi32(r, 0xd180aefeu));
+    p = madwide(rl, Q == 55 ? 0xb1721u : 0x2c5c86u, p);
     p -= mulwide(r, w) >> 13;
     return T - (mulhi64(T, p) >> 11);
 }
@@ -118,11 +137,10 @@ __host__ __device__ __forceinline__ uint64_t norm3(uint64_t x, uint64_t y, uint6
     y <<= sh;
     z <<= sh;
     const uint32_t xh = uint32_t(x >> 32), yh = uint32_t(y >> 32), zh = uint32_t(z >> 32);
-    // the three squares in units of 2^64: high parts and twice the cross
+    // the sum of squares in units of 2^64: high parts and twice the cross
     // terms (the squares of the low parts are below one unit)
-    const uint64_t H = mulwide(xh, xh) + mulwide(yh, yh) + mulwide(zh, zh);
-    const uint64_t C = mulwide(xh, uint32_t(x)) + mulwide(yh, uint32_t(y)) + mulwide(zh, uint32_t(z));
-    const uint64_t R = H + (C >> 31);  // in [2^58, 2^62)
+    const uint64_t C = madwide(xh, uint32_t(x), madwide(yh, uint32_t(y), mulwide(zh, uint32_t(z))));
+    const uint64_t R = madwide(xh, xh, madwide(yh, yh, madwide(zh, zh, C >> 31)));  // in [2^58, 2^62)
     const float f = float(uint32_t(R >> 32));
 #ifdef __CUDA_ARCH__
     float g;
@@ -136,8 +154,7 @@ __host__ __device__ __forceinline__ uint64_t norm3(uint64_t x, uint64_t y, uint6
     // sqrt(R) - r0 = e / (2 r0), in units of 2^-13
     const int32_t c = int32_t(float(int32_t(e >> 11)) * (g * 128.0f));
     // (R - (r0 + c 2^-13)^2) 2^26, exact modulo 2^64 and small
-    const int64_t e1 = int64_t(uint64_t(e) << 26) - int64_t(uint64_t(int64_t(int32_t(r0)) * c) << 14) -
-                       int64_t(c) * c;
+    const int64_t e1 = madwide_s(c, -c, int64_t((uint64_t(e) << 26) - (uint64_t(int64_t(int32_t(r0)) * c) << 14)));
     const int32_t c2 = int32_t(float(int32_t(e1 >> 18)) * (g * 128.0f));  // 2^-32
     const uint64_t r = (uint64_t(r0) << 32) + uint64_t(int64_t(c) * (1 << 19)) + uint64_t(int64_t(c2));
     return r >> sh;
@@ -152,9 +169,9 @@ __host__ __device__ __forceinline__ uint64_t exponent(uint64_t x, uint64_t y, ui
         // 2^-114 units -> 2^-53: drop 61 bits of the sum of squares
         const uint32_t xh = uint32_t(x >> 32), yh = uint32_t(y >> 32), zh = uint32_t(z >> 32);
         const uint32_t xl = uint32_t(x), yl = uint32_t(y), zl = uint32_t(z);
-        const uint64_t H = mulwide(xh, xh) + mulwide(yh, yh) + mulwide(zh, zh);
-        const uint64_t C = mulwide(xh, xl) + mulwide(yh, yl) + mulwide(zh, zl) +
-                           mulwide((mulhi32(xl, xl) >> 2) + (mulhi32(yl, yl) >> 2) + (mulhi32(zl, zl) >> 2), 2u);
+        const uint64_t H = madwide(xh, xh, madwide(yh, yh, mulwide(zh, zh)));
+        const uint64_t L = mulwide((mulhi32(xl, xl) >> 2) + (mulhi32(yl, yl) >> 2) + (mulhi32(zl, zl) >> 2), 2u);
+        const uint64_t C = madwide(xh, xl, madwide(yh, yl, madwide(zh, zl, L)));
         return (H << 3) + (C >> 28);
     }
     return norm3(x, y, z);
@@ -163,7 +180,7 @@ __host__ __device__ __forceinline__ uint64_t exponent(uint64_t x, uint64_t y, ui
 // 1 + t ln 2 (Matern-3/2), same units as t
 __host__ __device__ __forceinline__ uint64_t matern_factor(uint64_t t) {
     const uint32_t th = uint32_t(t >> 32), tl = uint32_t(t);
-    return (uint64_t(1) << 55) + mulwide(th, 0xb17217f7u) + mulhi32(th, 0xd1cf79acu) + mulhi32(tl, 0xb17217f7u);
+    return madwide(th, 0xb17217f7u, (uint64_t(1) << 55) + mulhi32(th, 0xd1cf79acu)) + mulhi32(tl, 0xb17217f7u);
 }
 
 // E 2^-63 2^-n as FP64 (n < 1000)

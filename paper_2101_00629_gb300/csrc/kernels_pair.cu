@@ -80,26 +80,52 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
 // 57-bit numbers relative to the largest of the group, in two limbs of 28 and
 // 29 bits, and three 32 x 32 -> 64-bit multiply-adds per column sum the group
 // exactly (the product of the two low limbs lies below the last bit kept).
-// One FP64 FMA per column and group adds the group to the running sum. The
-// error of a group is below 32 units of 2^-57 of its largest term; the groups
-// that take this path have values within a factor 2^9 of each other, so that
-// this stays below the rounding of an FP64 evaluation of the exponents.
+// One FP64 FMA per column and group adds the group to the running sum. A term
+// is off by 2^-58 of the group's largest value times its largest entry; an
+// FP64 evaluation rounds a value exp(-t ln 2) by (1.5 + t) 2^-53 of itself. The
+// groups that take this path have values within a factor 2^5 (1.5 + t) of each
+// other, t the largest exponent, so that even a group whose largest entry
+// meets its smallest value is no less exact than in FP64.
+//
+// A group is a block of the sources' tensor grid (SrcGrid), as near a cube as
+// the grid's spacing allows: 32 consecutive points of the half cylinder's
+// angle would span a third of it and leave most groups too wide.
 //
 // Each lane bounds the exponents of its targets against the box of the
 // group's source points, and the warp takes the first path that all its lanes
 // allow:
-//   products in integers   exponents within 9 of each other
+//   products in integers   exponents close to each other, as above
 //   products in FP64       exponents in the fixed-point range
 //   all in FP64            anything else: points too far apart for the range
 //                          (values below 2^-120 to 2^-1000), infinities, NaN,
 //                          entries below 2^-322
 //
 // Measured against the FP64 formula for every pair: 5003 x 20011 scattered
-// points, Matern-3/2, 3 columns, 8.13 -> 1.00 ms (integer products, issue
-// slots 64 % busy); half-cylinder Galerkin operator, Euclidean exponential,
-// 8 columns, 1.5e8 pairs, 10.7 -> 2.18 ms, and its degree-6 Gaussian
-// collocation operator, 3.7e8 pairs, 20.3 -> 5.1 ms (mostly FP64 products:
-// FP64 pipe 93 to 97 % busy).
+// points, Matern-3/2, 3 columns, 8.13 -> 0.84 ms; half-cylinder Galerkin
+// operator, Euclidean exponential, 8 columns, 1.5e8 pairs, 10.7 -> 1.59 ms, and
+// its degree-6 Gaussian collocation operator, 3.7e8 pairs, 20.3 -> 2.94 ms (with
+// groups of 32 consecutive points 2.18 and 5.1 ms: FP64 products, that pipe
+// 93 to 97 % busy). Bound by the integer pipes: 83 to 172 instructions per pair
+// and about seven per column, three of them 32 x 32 -> 64-bit multiply-adds of
+// four issue cycles. Two targets per thread were 5 to 20 % slower (registers).
+// Sources as a tensor grid n[0] x n[1] x n[2] (index i0 + n0 (i1 + n1 i2)) cut
+// into blocks of 2^s[0] x 2^s[1] x 2^s[2] points, 32 or fewer.
+struct SrcGrid {
+    int64_t n[3];
+    uint32_t nb[3];
+    int s[3];
+    __host__ __device__ int64_t groups() const { return int64_t(nb[0]) * nb[1] * nb[2]; }
+    // source of a lane of a group, -1 past the edge of the grid
+    __device__ int64_t source(uint32_t g, uint32_t lane) const {
+        const uint32_t g1 = g / nb[0], b0 = g - g1 * nb[0], b2 = g1 / nb[1], b1 = g1 - b2 * nb[1];
+        const int64_t i0 = (int64_t(b0) << s[0]) + (lane & ((1u << s[0]) - 1u));
+        const int64_t i1 = (int64_t(b1) << s[1]) + ((lane >> s[0]) & ((1u << s[1]) - 1u));
+        const int64_t i2 = (int64_t(b2) << s[2]) + ((lane >> (s[0] + s[1])) & ((1u << s[2]) - 1u));
+        const bool in = i0 < n[0] && i1 < n[1] && i2 < n[2] && (lane >> (s[0] + s[1] + s[2])) == 0;
+        return in ? i0 + n[0] * (i1 + n[1] * i2) : -1;
+    }
+};
+
 struct FxScale {
     uint64_t m;  // scale of a distance in base-2 exponents: m 2^e
     int e;
@@ -108,14 +134,14 @@ struct FxScale {
 
 __device__ const fx::Exp2Table g_exp2 = fx::Exp2Table();
 
-template <int KIND, int KB, int R>
-__global__ void __launch_bounds__(kTgt) pair_fx_kernel(
+template <int KIND, int KB>
+__global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     const double* __restrict__ tx, const double* __restrict__ ty, const double* __restrict__ tz,
     int64_t T, const double* __restrict__ sx, const double* __restrict__ sy,
-    const double* __restrict__ sz, int64_t S, const double* __restrict__ X, int64_t ldx, int k,
+    const double* __restrict__ sz, SrcGrid sg, const double* __restrict__ X, int64_t ldx, int k,
     int c0, double a, FxScale sc, double* __restrict__ part, int64_t per_split) {
-    constexpr int ST = KB > 8 ? 64 : 128;  // sources per stage
-    constexpr int NG = ST / 32;            // groups per stage
+    constexpr int NG = KB > 8 ? 2 : 4;  // groups per stage
+    constexpr int ST = 32 * NG;
     constexpr int Q = fx::Format<KIND>::kCoord, QA = fx::Format<KIND>::kArg;
     __shared__ __align__(16) uint64_t s_tab[2048];
     __shared__ __align__(16) uint64_t s_c[ST][4];
@@ -123,50 +149,47 @@ __global__ void __launch_bounds__(kTgt) pair_fx_kernel(
     __shared__ __align__(16) double s_xd[ST][KB];
     __shared__ float s_box[NG][6];
     __shared__ int s_emax[NG][KB];
-    __shared__ int s_special[NG];
+    __shared__ int s_special[NG], s_count[NG];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < 1024; i += kTgt)
         reinterpret_cast<ulonglong2*>(s_tab)[i] = reinterpret_cast<const ulonglong2*>(g_exp2.v)[i];
     const int split = blockIdx.y;
+    // groups [s0, s1) of this split
     const int64_t s0 = int64_t(split) * per_split;
-    const int64_t s1 = min(S, s0 + per_split);
-    const int64_t t0 = int64_t(blockIdx.x) * (kTgt * R);
+    const int64_t s1 = min(sg.groups(), s0 + per_split);
+    const int64_t t0 = int64_t(blockIdx.x) * kTgt;
     const int kc = min(KB, k - c0);
     // boxes are taken relative to the block's first target
     const double rx = tx[t0], ry = ty[t0], rz = tz[t0];
-    double px[R], py[R], pz[R];
-    uint64_t ux[R], uy[R], uz[R];
-    float fxr[R], fyr[R], fzr[R];
-    double acc[R][KB];
-    bool tfinite = true;
+    const int64_t tc = min(t0 + tid, T - 1);
+    const double px = tx[tc], py = ty[tc], pz = tz[tc];
+    const uint64_t ux = fx::to_fixed<Q>(px, sc.m, sc.e), uy = fx::to_fixed<Q>(py, sc.m, sc.e),
+                   uz = fx::to_fixed<Q>(pz, sc.m, sc.e);
+    const float p[3] = {float(px - rx) * sc.f, float(py - ry) * sc.f, float(pz - rz) * sc.f};
+    const bool tfinite = isfinite(p[0]) && isfinite(p[1]) && isfinite(p[2]);
+    double acc[KB];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int64_t t = min(t0 + r * kTgt + tid, T - 1);
-        px[r] = tx[t], py[r] = ty[t], pz[r] = tz[t];
-        ux[r] = fx::to_fixed<Q>(px[r], sc.m, sc.e);
-        uy[r] = fx::to_fixed<Q>(py[r], sc.m, sc.e);
-        uz[r] = fx::to_fixed<Q>(pz[r], sc.m, sc.e);
-        fxr[r] = float(px[r] - rx) * sc.f;
-        fyr[r] = float(py[r] - ry) * sc.f;
-        fzr[r] = float(pz[r] - rz) * sc.f;
-        tfinite = tfinite && isfinite(fxr[r]) && isfinite(fyr[r]) && isfinite(fzr[r]);
-#pragma unroll
-        for (int c = 0; c < KB; ++c) acc[r][c] = 0.0;
-    }
-    for (int64_t base = s0; base < s1; base += ST) {
-        const int n = int(s1 - base < ST ? s1 - base : int64_t(ST));
+    for (int c = 0; c < KB; ++c) acc[c] = 0.0;
+    for (int64_t base = s0; base < s1; base += NG) {
+        const int ng = int(s1 - base < NG ? s1 - base : int64_t(NG));
         __syncthreads();
-        // one warp per group of 32 sources, one source per lane; lanes past
-        // the end repeat the group's first source with zero entries
-        for (int g = warp; g < NG; g += kTgt / 32) {
-            if (g * 32 >= n) break;
-            const int j = g * 32 + lane;
-            const bool v = j < n;
-            const int64_t sj = base + (v ? j : g * 32);
-            const double x = sx[sj], y = sy[sj], z = sz[sj];
-            s_c[j][0] = fx::to_fixed<Q>(x, sc.m, sc.e);
-            s_c[j][1] = fx::to_fixed<Q>(y, sc.m, sc.e);
-            s_c[j][2] = fx::to_fixed<Q>(z, sc.m, sc.e);
+        // one warp per group, one source per lane; a block of the grid that
+        // reaches over its edge leaves lanes without a source, the others
+        // move together
+        for (int g = warp; g < ng; g += kTgt / 32) {
+            const int64_t sj = sg.source(uint32_t(base) + g, lane);
+            const unsigned have = __ballot_sync(0xffffffffu, sj >= 0);
+            const bool v = sj >= 0;
+            const int j = g * 32 + __popc(have & ((1u << lane) - 1u));
+            const int64_t sl = __shfl_sync(0xffffffffu, (long long)sj, __ffs(int(have)) - 1);
+            const int64_t sv = v ? sj : sl;
+            const double x = sx[sv], y = sy[sv], z = sz[sv];
+            if (v) {
+                s_c[j][0] = fx::to_fixed<Q>(x, sc.m, sc.e);
+                s_c[j][1] = fx::to_fixed<Q>(y, sc.m, sc.e);
+                s_c[j][2] = fx::to_fixed<Q>(z, sc.m, sc.e);
+                s_c[j][3] = uint64_t(sj);
+            }
             float lo[3] = {float(x - rx) * sc.f, float(y - ry) * sc.f, float(z - rz) * sc.f}, hi[3];
             bool bad = !(isfinite(lo[0]) && isfinite(lo[1]) && isfinite(lo[2]));
 #pragma unroll
@@ -181,7 +204,7 @@ __global__ void __launch_bounds__(kTgt) pair_fx_kernel(
 #pragma unroll
             for (int c = 0; c < KB; ++c) {
                 const double xv = (v && c < kc) ? X[sj + int64_t(c0 + c) * ldx] : 0.0;
-                s_xd[j][c] = xv;
+                if (v) s_xd[j][c] = xv;
                 const uint64_t b = uint64_t(__double_as_longlong(xv)) & 0x7fffffffffffffffull;
                 const int ef = int(b >> 52);
                 const int e = ef ? ef : (b ? 1 : 0);
@@ -195,137 +218,114 @@ __global__ void __launch_bounds__(kTgt) pair_fx_kernel(
                 if (rs <= 57) xi = int64_t((m + (rs ? uint64_t(1) << (rs - 1) : 0)) >> rs);
                 if (xv < 0.0) xi = -xi;
                 const int32_t x1 = int32_t((xi + (1 << 27)) >> 28);
-                s_xl[j][c] = make_int2(x1, int32_t(xi - (int64_t(x1) << 28)));
+                if (v) s_xl[j][c] = make_int2(x1, int32_t(xi - (int64_t(x1) << 28)));
                 if (lane == 0) s_emax[g][c] = emax;
             }
             const bool any_bad = __any_sync(0xffffffffu, bad);
             if (lane == 0) {
                 s_special[g] = any_bad;
+                s_count[g] = __popc(have);
 #pragma unroll
                 for (int q = 0; q < 3; ++q) s_box[g][q] = lo[q], s_box[g][3 + q] = hi[q];
             }
         }
         __syncthreads();
-        for (int g = 0; g * 32 < n; ++g) {
-            const int j0 = g * 32, j1 = min(n, j0 + 32);
+        for (int g = 0; g < ng; ++g) {
+            const int j0 = g * 32, j1 = j0 + s_count[g];
             // bounds of the exponents over the box; the slack covers the
             // rounding of the single-precision coordinates
-            int n0[R], gm[R];
-            bool in_range = tfinite && !s_special[g], narrow = true;
+            float tlo = 0.0f, thi = 0.0f;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float p[3] = {fxr[r], fyr[r], fzr[r]};
-                float tlo = 0.0f, thi = 0.0f;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const float lo = s_box[g][q], hi = s_box[g][3 + q];
-                    const float eps = 1e-6f * (fabsf(lo) + fabsf(hi) + fabsf(p[q]));
-                    const float dl = fmaxf(fmaxf(lo - p[q], p[q] - hi) - eps, 0.0f);
-                    const float dh = fmaxf(p[q] - lo, hi - p[q]) + eps;
-                    tlo += KIND == KL_KERNEL_EXP_SEP ? dl : dl * dl;
-                    thi += KIND == KL_KERNEL_EXP_SEP ? dh : dh * dh;
-                }
-                if (KIND == KL_KERNEL_EXP || KIND == KL_KERNEL_MATERN32) {
-                    tlo = sqrtf(tlo);
-                    thi = sqrtf(thi);
-                }
-                in_range = in_range && thi < fx::Format<KIND>::kMaxArg;
-                gm[r] = 0;
-                if (KIND == KL_KERNEL_MATERN32) {
-                    const float fh = 1.0f + 0.6931472f * thi;
-                    gm[r] = 1 + int(log2f(fh) + 1e-3f);  // 1 + t ln 2 < 2^gm
-                    tlo -= log2f(1.0f + 0.6931472f * tlo);
-                    thi -= log2f(fh);
-                }
-                tlo = fmaxf(tlo * (1.0f - 1e-5f) - 1e-3f, 0.0f);
-                thi = thi * (1.0f + 1e-5f) + 1e-3f;
-                n0[r] = int(fminf(tlo, 1000.0f));
-                narrow = narrow && thi - float(n0[r]) < 9.0f;
+            for (int q = 0; q < 3; ++q) {
+                const float lo = s_box[g][q], hi = s_box[g][3 + q];
+                const float eps = 1e-6f * (fabsf(lo) + fabsf(hi) + fabsf(p[q]));
+                const float dl = fmaxf(fmaxf(lo - p[q], p[q] - hi) - eps, 0.0f);
+                const float dh = fmaxf(p[q] - lo, hi - p[q]) + eps;
+                tlo += KIND == KL_KERNEL_EXP_SEP ? dl : dl * dl;
+                thi += KIND == KL_KERNEL_EXP_SEP ? dh : dh * dh;
             }
+            if (KIND == KL_KERNEL_EXP || KIND == KL_KERNEL_MATERN32) {
+                tlo = sqrtf(tlo);
+                thi = sqrtf(thi);
+            }
+            const bool in_range = tfinite && !s_special[g] && thi < fx::Format<KIND>::kMaxArg;
+            const float most = 5.0f + log2f(1.5f + thi);
+            int gm = 0;
+            if (KIND == KL_KERNEL_MATERN32) {
+                const float fh = 1.0f + 0.6931472f * thi;
+                gm = 1 + int(log2f(fh) + 1e-3f);  // 1 + t ln 2 < 2^gm
+                tlo -= log2f(1.0f + 0.6931472f * tlo);
+                thi -= log2f(fh);
+            }
+            tlo = fmaxf(tlo * (1.0f - 1e-5f) - 1e-3f, 0.0f);
+            thi = thi * (1.0f + 1e-5f) + 1e-3f;
+            const int n0 = int(fminf(tlo, 1000.0f));
+            const bool narrow = thi - float(n0) < most;
             if (__all_sync(0xffffffffu, in_range && narrow)) {
-                int64_t hi[R][KB], mid[R][KB];
+                int64_t hi[KB], mid[KB];
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int c = 0; c < KB; ++c) hi[r][c] = 0, mid[r][c] = 0;
+                for (int c = 0; c < KB; ++c) hi[c] = 0, mid[c] = 0;
+#pragma unroll 2
                 for (int j = j0; j < j1; ++j) {
-                    uint32_t g1[R], g0[R];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const uint64_t t = fx::exponent<KIND>(fx::absdiff(ux[r], s_c[j][0]),
-                                                              fx::absdiff(uy[r], s_c[j][1]),
-                                                              fx::absdiff(uz[r], s_c[j][2]));
-                        uint32_t nt;
-                        uint64_t E = fx::exp2_neg<QA>(t, s_tab, nt);
-                        if (KIND == KL_KERNEL_MATERN32) {
-                            const uint64_t W = fx::matern_factor(t) << (9 - gm[r]);
-                            E = fx::mulhi64(E, W) >> (6 + int(nt) - n0[r] - gm[r]);
-                            g1[r] = uint32_t(E >> 28);
-                            g0[r] = uint32_t(E) & 0xfffffffu;
-                        } else {
-                            const uint32_t s = 2u + nt - uint32_t(n0[r]);
-                            g1[r] = uint32_t(E >> 32) >> s;
-                            g0[r] = __funnelshift_r(uint32_t(E), uint32_t(E >> 32), s) >> 4;
-                        }
+                    const ulonglong2 qxy = *reinterpret_cast<const ulonglong2*>(s_c[j]);
+                    const uint64_t t = fx::exponent<KIND>(fx::absdiff(ux, qxy.x), fx::absdiff(uy, qxy.y),
+                                                          fx::absdiff(uz, s_c[j][2]));
+                    uint32_t nt, g1, g0;
+                    uint64_t E = fx::exp2_neg<QA>(t, s_tab, nt);
+                    if (KIND == KL_KERNEL_MATERN32) {
+                        E = fx::mulhi64(E, fx::matern_factor(t) << (9 - gm)) >> (6 + int(nt) - n0 - gm);
+                        g1 = uint32_t(E >> 28);
+                        g0 = uint32_t(E) & 0xfffffffu;
+                    } else {
+                        const uint32_t s = 2u + nt - uint32_t(n0);
+                        g1 = uint32_t(E >> 32) >> s;
+                        g0 = __funnelshift_r(uint32_t(E), uint32_t(E >> 32), s) >> 4;
                     }
 #pragma unroll
                     for (int c = 0; c < KB; ++c) {
-                        const int2 xl = s_xl[j][c];
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            hi[r][c] += int64_t(int32_t(g1[r])) * xl.x;
-                            mid[r][c] += int64_t(int32_t(g1[r])) * xl.y;
-                            mid[r][c] += int64_t(int32_t(g0[r])) * xl.x;
+                        int2 xl;  // two columns per 16-byte load
+                        if (KB == 1) {
+                            xl = s_xl[j][c];
+                        } else {
+                            const int4 x2 = *reinterpret_cast<const int4*>(&s_xl[j][c & ~1]);
+                            xl = c & 1 ? make_int2(x2.z, x2.w) : make_int2(x2.x, x2.y);
                         }
+                        hi[c] = fx::madwide_s(int32_t(g1), xl.x, hi[c]);
+                        mid[c] = fx::madwide_s(int32_t(g1), xl.y, mid[c]);
+                        mid[c] = fx::madwide_s(int32_t(g0), xl.x, mid[c]);
                     }
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int c = 0; c < KB; ++c) {
-                        const int64_t sum = hi[r][c] + (mid[r][c] >> 28);
-                        const double f = __longlong_as_double((long long)(s_emax[g][c] - 56 - n0[r]) << 52);
-                        acc[r][c] = fma(double(sum), f, acc[r][c]);
-                    }
+                for (int c = 0; c < KB; ++c) {
+                    const int64_t sum = hi[c] + (mid[c] >> 28);
+                    const double f = __longlong_as_double((long long)(s_emax[g][c] - 56 - n0) << 52);
+                    acc[c] = fma(double(sum), f, acc[c]);
+                }
             } else if (__all_sync(0xffffffffu, in_range)) {
                 for (int j = j0; j < j1; ++j) {
-                    double gv[R];
+                    const uint64_t t = fx::exponent<KIND>(fx::absdiff(ux, s_c[j][0]), fx::absdiff(uy, s_c[j][1]),
+                                                          fx::absdiff(uz, s_c[j][2]));
+                    uint32_t nt;
+                    const uint64_t E = fx::exp2_neg<QA>(t, s_tab, nt);
+                    double gv = fx::to_double(E, nt);
+                    if (KIND == KL_KERNEL_MATERN32) gv *= double(fx::matern_factor(t)) * 2.7755575615628914e-17;  // 2^-55
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const uint64_t t = fx::exponent<KIND>(fx::absdiff(ux[r], s_c[j][0]),
-                                                              fx::absdiff(uy[r], s_c[j][1]),
-                                                              fx::absdiff(uz[r], s_c[j][2]));
-                        uint32_t nt;
-                        const uint64_t E = fx::exp2_neg<QA>(t, s_tab, nt);
-                        gv[r] = fx::to_double(E, nt);
-                        if (KIND == KL_KERNEL_MATERN32)
-                            gv[r] *= double(fx::matern_factor(t)) * 2.7755575615628914e-17;  // 2^-55
-                    }
-#pragma unroll
-                    for (int c = 0; c < KB; ++c)
-#pragma unroll
-                        for (int r = 0; r < R; ++r) acc[r][c] = fma(gv[r], s_xd[j][c], acc[r][c]);
+                    for (int c = 0; c < KB; ++c) acc[c] = fma(gv, s_xd[j][c], acc[c]);
                 }
             } else {
                 for (int j = j0; j < j1; ++j) {
-                    const double qx = sx[base + j], qy = sy[base + j], qz = sz[base + j];
+                    const int64_t sj = int64_t(s_c[j][3]);
+                    const double gv = gamma64<KIND>(px - sx[sj], py - sy[sj], pz - sz[sj], a);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double gv = gamma64<KIND>(px[r] - qx, py[r] - qy, pz[r] - qz, a);
-#pragma unroll
-                        for (int c = 0; c < KB; ++c) acc[r][c] = fma(gv, s_xd[j][c], acc[r][c]);
-                    }
+                    for (int c = 0; c < KB; ++c) acc[c] = fma(gv, s_xd[j][c], acc[c]);
                 }
             }
         }
     }
+    if (t0 + tid < T) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int64_t t = t0 + r * kTgt + tid;
-        if (t < T)
-#pragma unroll
-            for (int c = 0; c < KB; ++c)
-                if (c < kc) part[(int64_t(split) * k + c0 + c) * T + t] = acc[r][c];
+        for (int c = 0; c < KB; ++c)
+            if (c < kc) part[(int64_t(split) * k + c0 + c) * T + t0 + tid] = acc[c];
     }
 }
 
@@ -431,20 +431,45 @@ void launch_f64(const PairArgs& a, int c0, int64_t per_split, cudaStream_t s) {
         pair_f64_kernel<KIND, 32><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
 }
 
+// Blocks of the source grid: from one point, double the block along the
+// direction in which it is shortest until it has 32; fewer (down to 4) where
+// the splits would outnumber the blocks.
+SrcGrid src_grid(const PairArgs& a) {
+    SrcGrid g{};
+    for (int bits = 5; bits >= 2; --bits) {
+        double h[3];
+        for (int d = 0; d < 3; ++d) {
+            g.n[d] = a.sn[0] > 0 ? a.sn[d] : (d == 0 ? a.S : 1);
+            h[d] = a.sn[0] > 0 ? a.sh[d] : 1.0;
+            g.s[d] = 0;
+        }
+        for (int left = bits; left > 0; --left) {
+            int best = -1;
+            for (int d = 0; d < 3; ++d)
+                if ((int64_t(1) << g.s[d]) < g.n[d] && (best < 0 || h[d] < h[best])) best = d;
+            if (best < 0) break;
+            ++g.s[best];
+            h[best] *= 2.0;
+        }
+        for (int d = 0; d < 3; ++d) g.nb[d] = uint32_t((g.n[d] + (int64_t(1) << g.s[d]) - 1) >> g.s[d]);
+        if (g.groups() >= a.splits) break;
+    }
+    return g;
+}
+
 template <int KIND>
-void launch_fx(const PairArgs& a, int c0, int64_t per_split, const FxScale& sc, cudaStream_t s) {
+void launch_fx(const PairArgs& a, int c0, const FxScale& sc, const SrcGrid& sg, cudaStream_t s) {
     const int kc = a.k - c0;
-    auto go = [&](auto kb, auto r) {
-        constexpr int KB = decltype(kb)::value, R = decltype(r)::value;
-        const dim3 grid(unsigned((a.T + kTgt * R - 1) / (kTgt * R)), unsigned(a.splits));
-        pair_fx_kernel<KIND, KB, R><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, sc, a.scratch, per_split);
+    const int64_t per_split = (sg.groups() + a.splits - 1) / a.splits;
+    const dim3 grid(unsigned((a.T + kTgt - 1) / kTgt), unsigned(a.splits));
+    auto go = [&](auto kb) {
+        pair_fx_kernel<KIND, decltype(kb)::value><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, sg, a.X, a.ldx, a.k, c0, a.ks.a, sc, a.scratch, per_split);
     };
-    using I1 = std::integral_constant<int, 1>;
-    if (kc <= 1) go(I1{}, I1{});
-    else if (kc <= 2) go(std::integral_constant<int, 2>{}, I1{});
-    else if (kc <= 4) go(std::integral_constant<int, 4>{}, I1{});
-    else if (kc <= 8) go(std::integral_constant<int, 8>{}, I1{});
-    else go(std::integral_constant<int, 16>{}, I1{});
+    if (kc <= 1) go(std::integral_constant<int, 1>{});
+    else if (kc <= 2) go(std::integral_constant<int, 2>{});
+    else if (kc <= 4) go(std::integral_constant<int, 4>{});
+    else if (kc <= 8) go(std::integral_constant<int, 8>{});
+    else go(std::integral_constant<int, 16>{});
 }
 
 template <int KIND>
@@ -472,6 +497,7 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
     dim3 grid(unsigned((a.T + kTgt - 1) / kTgt), unsigned(a.splits));
     const double l2e = 1.4426950408889634074;
     const FxScale sc = fx_scale(KIND, a.ks.a);
+    const SrcGrid sg = src_grid(a);
     // columns per pass over the pairs: 32, in fixed point 16 (two 64-bit
     // sums per column in registers)
     const int step = fp32 || KIND == KL_KERNEL_CONST ? 32 : 16;
@@ -489,7 +515,7 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
             if constexpr (KIND == KL_KERNEL_CONST) {
                 launch_f64<KIND>(a, c0, per_split, s);
             } else {
-                launch_fx<KIND>(a, c0, per_split, sc, s);
+                launch_fx<KIND>(a, c0, sc, sg, s);
             }
         }
         cudaError_t e = cudaGetLastError();

@@ -154,6 +154,10 @@ struct PairArgs {
     const double *sx, *sy, *sz;  // sources (S), FP64
     const float *sx32, *sy32, *sz32;
     int64_t T, S;
+    // sources as a tensor grid, direction 1 fastest: points and mean spacing
+    // per direction (sn[0] = 0: scattered points)
+    int sn[3];
+    double sh[3];
     const double* X;  // S x k (ldx)
     int64_t ldx;
     double* Y;  // T x k (ldy)
