@@ -129,6 +129,9 @@ void domain_extent(const kl_params& p, double* e) {
     }
 }
 
+// Precisions whose pairwise product runs on the CUDA cores.
+bool cuda_cores(int precision) { return precision == KL_FP64 || precision == KL_FP32; }
+
 template <class T>
 cudaError_t dalloc(kl_solver* h, T** p, int64_t count) {
     *p = nullptr;
@@ -163,7 +166,7 @@ int ensure_workspace(kl_solver* h, int k) {
     const int64_t big = std::max(h->S, h->T) * int64_t(k);
     for (int i = 0; i < 3; ++i)
         if ((e = dalloc(h, &h->ws[i], big)) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
-    h->pair_splits = pair_choose_splits(h->T, h->S, h->sm_count);
+    h->pair_splits = pair_choose_splits(h->T, h->S, h->sm_count, cuda_cores(h->prm.precision));
     h->pair_scratch_len = std::max<int64_t>(pair_scratch_doubles(h->T, k, h->pair_splits),
                                             tc_scratch_doubles(h->T, h->S, k, h->sm_count));
     if ((e = dalloc(h, &h->pair_scratch, h->pair_scratch_len)) != cudaSuccess)
@@ -1033,7 +1036,7 @@ int kl_estimate_bytes(const kl_params* params, int M, int64_t* bytes) {
     const int64_t points = (gal ? 4 * S : 3 * T + 4 * S) + (3 * T + 3 * S + 1) / 2 + 1 +
                            (p.geometry == KL_GEOM_PROJECTIVE_CUBE && !gal ? 3 * N + 2 * S : 0);
     const int64_t ws = 3 * std::max(S, T) * int64_t(kmax);
-    const int64_t pair = std::max<int64_t>(pair_scratch_doubles(T, kmax, pair_choose_splits(T, S, sm)),
+    const int64_t pair = std::max<int64_t>(pair_scratch_doubles(T, kmax, pair_choose_splits(T, S, sm, cuda_cores(p.precision))),
                                            tc_scratch_doubles(T, S, kmax, sm));
     const int64_t eig = eig_workspace_doubles(N, mcap);
     const int64_t total = 8 * (tab + points + ws + pair + eig);

@@ -329,65 +329,121 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     }
 }
 
-template <int KIND, int KB>
+// FP32 product: R targets per thread, so that a source's coordinates (one
+// 16-byte load) and its KB entries serve R pairs. Bound by instruction issue:
+// about 12 per value (two of them special-function), KB per product, and by
+// the FP64 additions of the tile sums. 2688 x 82368 points, Matern-3/2, whole
+// application: 5 columns 249 -> 205 us, 16 columns 455 -> 410 us against one
+// target per thread, scalar coordinate loads and 8 columns at least.
+template <int KIND, int KB, int R>
 __global__ void __launch_bounds__(kTgt) pair_f32_kernel(
     const float* __restrict__ tx, const float* __restrict__ ty, const float* __restrict__ tz,
     int64_t T, const float* __restrict__ sx, const float* __restrict__ sy,
     const float* __restrict__ sz, int64_t S, const double* __restrict__ X, int64_t ldx, int k,
     int c0, float a, float a2, double* __restrict__ part, int64_t per_split) {
-    __shared__ float s_x[kSrc], s_y[kSrc], s_z[kSrc];
-    __shared__ float s_v[kSrc][KB];
-    const int64_t t = int64_t(blockIdx.x) * kTgt + threadIdx.x;
+    __shared__ float4 s_c[kSrc];
+    __shared__ __align__(16) float s_v[kSrc][KB];
+    const int64_t t0 = int64_t(blockIdx.x) * (kTgt * R) + threadIdx.x;
     const int split = blockIdx.y;
     const int64_t s0 = int64_t(split) * per_split;
     const int64_t s1 = min(S, s0 + per_split);
-    const float px = t < T ? tx[t] : 0.f, py = t < T ? ty[t] : 0.f, pz = t < T ? tz[t] : 0.f;
-    const int kc = min(KB, k - c0);
-    float acc[KB];
-    double accd[KB];
+    float px[R], py[R], pz[R];
 #pragma unroll
-    for (int c = 0; c < KB; ++c) acc[c] = 0.f, accd[c] = 0.0;
+    for (int r = 0; r < R; ++r) {
+        const int64_t t = t0 + r * kTgt;
+        px[r] = t < T ? tx[t] : 0.f, py[r] = t < T ? ty[t] : 0.f, pz[r] = t < T ? tz[t] : 0.f;
+    }
+    const int kc = min(KB, k - c0);
+    float acc[R][KB];
+    double accd[R][KB];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < KB; ++c) acc[r][c] = 0.f, accd[r][c] = 0.0;
     for (int64_t base = s0; base < s1; base += kSrc) {
         const int n = int(s1 - base < kSrc ? s1 - base : int64_t(kSrc));
         __syncthreads();
         for (int i = threadIdx.x; i < kSrc; i += kTgt) {
             const bool v = i < n;
-            s_x[i] = v ? sx[base + i] : 0.f;
-            s_y[i] = v ? sy[base + i] : 0.f;
-            s_z[i] = v ? sz[base + i] : 0.f;
+            s_c[i] = v ? make_float4(sx[base + i], sy[base + i], sz[base + i], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int i = threadIdx.x; i < kSrc * KB; i += kTgt) {
             const int c = i / kSrc, j = i - c * kSrc;
             s_v[j][c] = (j < n && c < kc) ? float(X[base + j + int64_t(c0 + c) * ldx]) : 0.f;
         }
         __syncthreads();
+#pragma unroll 2
         for (int j = 0; j < n; ++j) {
-            const float g = gamma32<KIND>(px - s_x[j], py - s_y[j], pz - s_z[j], a, a2);
+            const float4 q = s_c[j];
+            float g[R];
 #pragma unroll
-            for (int c = 0; c < KB; ++c) acc[c] = fmaf(g, s_v[j][c], acc[c]);
+            for (int r = 0; r < R; ++r) g[r] = gamma32<KIND>(px[r] - q.x, py[r] - q.y, pz[r] - q.z, a, a2);
+#pragma unroll
+            for (int c = 0; c < KB; ++c) {
+                const float v = s_v[j][c];
+#pragma unroll
+                for (int r = 0; r < R; ++r) acc[r][c] = fmaf(g[r], v, acc[r][c]);
+            }
         }
         // flush the FP32 tile sums into FP64 once per tile
 #pragma unroll
-        for (int c = 0; c < KB; ++c) accd[c] += double(acc[c]), acc[c] = 0.f;
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < KB; ++c) accd[r][c] += double(acc[r][c]), acc[r][c] = 0.f;
     }
-    if (t < T) {
-        for (int c = 0; c < kc; ++c) part[(int64_t(split) * k + c0 + c) * T + t] = accd[c];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int64_t t = t0 + r * kTgt;
+        if (t < T) {
+#pragma unroll
+            for (int c = 0; c < KB; ++c)
+                if (c < kc) part[(int64_t(split) * k + c0 + c) * T + t] = accd[r][c];
+        }
     }
 }
 
-__global__ void pair_reduce_kernel(const double* __restrict__ part, int splits, int64_t T, int k,
-                                   double sigma2, const double* __restrict__ post, double* Y,
-                                   int64_t ldy) {
-    const int64_t total = T * k;
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < total;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t c = i / T, t = i - c * T;
+// Y = sigma^2 post .* (sum of the splits' partial sums). A block serves 32
+// points of one column, warp y the y-th eighth of the splits; warp 0 adds the
+// eight in order. With one thread per output, 64 loads one after the other
+// took 15 to 20 us (cold) for a few thousand points.
+constexpr int kRedSlices = 8;
+__global__ void __launch_bounds__(32 * kRedSlices) pair_reduce_kernel(const double* __restrict__ part, int splits,
+                                                                      int64_t T, int k, double sigma2,
+                                                                      const double* __restrict__ post, double* Y,
+                                                                      int64_t ldy) {
+    __shared__ double sh[kRedSlices][32];
+    const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+    const int per = (splits + kRedSlices - 1) / kRedSlices;
+    const int sp0 = min(splits, sl * per), sp1 = min(splits, sp0 + per);
+    const int64_t tiles = (T + 31) / 32;
+    for (int64_t b = blockIdx.x; b < tiles * k; b += gridDim.x) {
+        const int64_t c = b / tiles, t = (b - c * tiles) * 32 + lane;
         double s = 0.0;
-        for (int sp = 0; sp < splits; ++sp) s += part[(int64_t(sp) * k + c) * T + t];
-        s *= sigma2;
-        if (post) s *= post[t];
-        Y[c * ldy + t] = s;
+        if (t < T) {
+            const double* p = part + c * T + t;
+            const int64_t step = int64_t(k) * T;
+#pragma unroll 8
+            for (int sp = sp0; sp < sp1; ++sp) s += p[sp * step];
+        }
+        __syncthreads();
+        sh[sl][lane] = s;
+        __syncthreads();
+        if (sl == 0 && t < T) {
+#pragma unroll
+            for (int q = 1; q < kRedSlices; ++q) s += sh[q][lane];
+            s *= sigma2;
+            if (post) s *= post[t];
+            Y[c * ldy + t] = s;
+        }
     }
+}
+
+cudaError_t run_pair_reduce(const double* part, int splits, int64_t T, int k, double sigma2, const double* post,
+                            double* Y, int64_t ldy, cudaStream_t s) {
+    const int64_t blocks = (T + 31) / 32 * k;
+    const int g = int(std::min<int64_t>(blocks, int64_t(device_sm_count()) * 32));
+    pair_reduce_kernel<<<g < 1 ? 1 : g, 32 * kRedSlices, 0, s>>>(part, splits, T, k, sigma2, post, Y, ldy);
+    return cudaGetLastError();
 }
 
 // Scale of a distance (Gauss: its square root is taken) in base-2 exponents,
@@ -494,7 +550,6 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
     KL_RANGE(a.scratch, pair_scratch_doubles(a.T, a.k, a.splits), double, "pair partial sums");
     KL_RANGE(a.Y, block_extent(a.T, a.k, a.ldy), double, "pair Y");
     KL_RANGE(a.post, a.T, double, "pair post");
-    dim3 grid(unsigned((a.T + kTgt - 1) / kTgt), unsigned(a.splits));
     const double l2e = 1.4426950408889634074;
     const FxScale sc = fx_scale(KIND, a.ks.a);
     const SrcGrid sg = src_grid(a);
@@ -505,12 +560,18 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
         const int kc = a.k - c0;
         if (fp32) {
             const float fa = float(a.ks.a), fa2 = float(a.ks.a * l2e);
-            if (kc <= 8)
-                pair_f32_kernel<KIND, 8><<<grid, kTgt, 0, s>>>(a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
-            else if (kc <= 16)
-                pair_f32_kernel<KIND, 16><<<grid, kTgt, 0, s>>>(a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
-            else
-                pair_f32_kernel<KIND, 32><<<grid, kTgt, 0, s>>>(a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
+            auto go = [&](auto kb, auto r) {
+                constexpr int KB = decltype(kb)::value, R = decltype(r)::value;
+                const dim3 grid(unsigned((a.T + kTgt * R - 1) / (kTgt * R)), unsigned(a.splits));
+                pair_f32_kernel<KIND, KB, R><<<grid, kTgt, 0, s>>>(a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
+            };
+            using I1 = std::integral_constant<int, 1>;
+            using I2 = std::integral_constant<int, 2>;
+            if (kc <= 4) go(std::integral_constant<int, 4>{}, I2{});
+            else if (kc <= 6) go(std::integral_constant<int, 6>{}, I2{});
+            else if (kc <= 8) go(std::integral_constant<int, 8>{}, I2{});
+            else if (kc <= 16) go(std::integral_constant<int, 16>{}, I2{});
+            else go(std::integral_constant<int, 32>{}, I1{});
         } else {
             if constexpr (KIND == KL_KERNEL_CONST) {
                 launch_f64<KIND>(a, c0, per_split, s);
@@ -521,38 +582,23 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    const int64_t total = a.T * a.k;
-    int g = int(std::min<int64_t>((total + 255) / 256, int64_t(device_sm_count()) * 32));
-    pair_reduce_kernel<<<g < 1 ? 1 : g, 256, 0, s>>>(a.scratch, a.splits, a.T, a.k, a.ks.sigma2, a.post, a.Y, a.ldy);
-    return cudaGetLastError();
+    return run_pair_reduce(a.scratch, a.splits, a.T, a.k, a.ks.sigma2, a.post, a.Y, a.ldy, s);
 }
 
 }  // namespace
 
 int64_t pair_scratch_doubles(int64_t T, int k, int splits) { return T * int64_t(k) * splits; }
 
-int pair_choose_splits(int64_t T, int64_t S, int sm_count) {
+int pair_choose_splits(int64_t T, int64_t S, int sm_count, bool fine) {
+    // 16 blocks per SM while a split keeps 512 sources. `fine`: 256, and few
+    // sources are cut down to 16 per split for one wave of five blocks per SM
+    // (216 targets and sources, one column, FP64: 250 us in one split per tile
+    // of targets, 12 us in 13); the partial sums take more memory, which
+    // handles that use this product for a refinement only do without.
     const int64_t tb = (T + kTgt - 1) / kTgt;
-    int64_t want = (16LL * sm_count + tb - 1) / tb;
-    // at least 16 sources per split: 216 targets and sources (one column,
-    // FP64) took 250 us in one split per tile of targets, 16 us in 13
-    int64_t cap = S / 16;
-    if (cap < 1) cap = 1;
-    if (want > cap) want = cap;
-    if (want < 1) want = 1;
-    if (want > 64) want = 64;
-    return int(want);
-}
-
-cudaError_t launch_pair_reduce(const double* part, int splits, int64_t T, int k, double sigma2,
-                               const double* post, double* Y, int64_t ldy, cudaStream_t s) {
-    KL_RANGE(part, pair_scratch_doubles(T, k, splits), double, "pair_reduce partial sums");
-    KL_RANGE(Y, block_extent(T, k, ldy), double, "pair_reduce Y");
-    KL_RANGE(post, T, double, "pair_reduce post");
-    const int64_t total = T * k;
-    int g = int(std::min<int64_t>((total + 255) / 256, int64_t(device_sm_count()) * 32));
-    pair_reduce_kernel<<<g < 1 ? 1 : g, 256, 0, s>>>(part, splits, T, k, sigma2, post, Y, ldy);
-    return cudaGetLastError();
+    const int64_t many = std::min<int64_t>((16LL * sm_count + tb - 1) / tb, S / (fine ? 256 : 512));
+    const int64_t few = fine ? std::min<int64_t>(5LL * sm_count / tb, S / 16) : 1;
+    return int(std::min<int64_t>(64, std::max<int64_t>(1, std::max(many, few))));
 }
 
 cudaError_t launch_pair_simt(const PairArgs& a, bool fp32, cudaStream_t s) {

@@ -113,8 +113,4 @@ cudaError_t tc_sym_upload(const TcSymPlan& p, double* scratch, cudaStream_t s);
 // Conversion, one tcgen05 launch and one ordered reduction per band.
 cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched);
 
-// Reduction of split partials shared with the CUDA-core kernels.
-cudaError_t launch_pair_reduce(const double* part, int splits, int64_t T, int k, double sigma2,
-                               const double* post, double* Y, int64_t ldy, cudaStream_t s);
-
 }  // namespace kl

@@ -169,7 +169,7 @@ struct PairArgs {
     int splits;
 };
 int64_t pair_scratch_doubles(int64_t T, int k, int splits);
-int pair_choose_splits(int64_t T, int64_t S, int sm_count);
+int pair_choose_splits(int64_t T, int64_t S, int sm_count, bool fine);
 cudaError_t launch_pair_simt(const PairArgs& a, bool fp32, cudaStream_t s);
 
 // ---------------------------------------------------------------------------

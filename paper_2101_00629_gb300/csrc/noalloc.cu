@@ -78,7 +78,7 @@ extern "C" int kl_pairwise_noalloc(int kernel, double sigma, double L, const dou
     int sms = 0;
     int rc = device_scratch(&scratch, &sms);
     if (rc != KL_OK) return rc;
-    int splits = pair_choose_splits(T, S, sms);
+    int splits = pair_choose_splits(T, S, sms, true);
     const int64_t cap = kNoallocScratch / (int64_t(k) * T);
     if (splits > cap) splits = int(cap);
     PairArgs a{};
