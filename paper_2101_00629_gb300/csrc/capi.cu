@@ -340,7 +340,7 @@ static int pairwise(kl_solver* h, int precision, const double* U, double* W, int
             e = h->batcher->run(job);
         }
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, job.done, 0);
-        if (e == cudaSuccess) e = tc_finish(a, h->stream, &launched);
+        if (e == cudaSuccess) e = tc_finish(a, h->stream, &launched, false);
         h->launches += launched + 1;
         if (e != cudaSuccess) return cuda_fail(h, e, "pairwise (tcgen05, batched)");
         return KL_OK;

@@ -746,6 +746,7 @@ __global__ void __launch_bounds__(kEigThreads) nonsym_eig_kernel(const double* _
                                                                  double* Vout, double* Qout, double* work_d,
                                                                  int* status, int smem_level, int sym,
                                                                  int nvec) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* smem_a = reinterpret_cast<R*>(smem_raw);
     R* work = reinterpret_cast<R*>(work_d);
@@ -1559,7 +1560,7 @@ cudaError_t launch_eig_t(const double* H, int n, double* wr, double* wi, double*
                                           int(kEigSmemLimit));
     });
     if (attr_error != cudaSuccess) return attr_error;
-    nonsym_eig_kernel<R><<<1, kEigThreads, bytes, s>>>(H, n, wr, wi, V, Q, work, status, level, sym, nvec);
+    launch_chain(nonsym_eig_kernel<R>, 1, kEigThreads, bytes, s, H, n, wr, wi, V, Q, work, status, level, sym, nvec);
     return cudaGetLastError();
 }
 

@@ -75,6 +75,7 @@ template <class R>
 __global__ void __launch_bounds__(kJacThreads) jacobi_kernel(const double* __restrict__ H, int n, int max_sweeps,
                                                             double* __restrict__ w, double* __restrict__ V,
                                                             int* __restrict__ status) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char jac_smem[];
     const int ld = n + 1;
     R* A = reinterpret_cast<R*>(jac_smem);  // A[i * ld + j] = H(i, j)
@@ -207,7 +208,7 @@ cudaError_t launch_jacobi(const double* H, int n, int max_sweeps, double* w, dou
                                           int(jacobi_smem_bytes(kJacMaxN, sizeof(R))));
     });
     if (attr_error != cudaSuccess) return attr_error;
-    jacobi_kernel<R><<<1, kJacThreads, jacobi_smem_bytes(n, sizeof(R)), s>>>(H, n, max_sweeps, w, V, status);
+    launch_chain(jacobi_kernel<R>, 1, kJacThreads, jacobi_smem_bytes(n, sizeof(R)), s, H, n, max_sweeps, w, V, status);
     return cudaGetLastError();
 }
 

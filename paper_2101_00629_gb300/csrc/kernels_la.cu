@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256) gemm_tn_kernel(const double* __restrict__
                                                       const double* __restrict__ B, int64_t ldb,
                                                       int m, int n, int64_t K, int64_t kchunk,
                                                       double* __restrict__ part) {
+    chain_wait();
     __shared__ double As[TN_T][TN_T + 1];
     __shared__ double Bs[TN_T][TN_T + 1];
     const int i0 = blockIdx.x * TN_T, j0 = blockIdx.y * TN_T;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(256) gemm_tn_narrow_kernel(const double* __res
                                                              const double* __restrict__ B, int64_t ldb,
                                                              int m, int n, int64_t K, int64_t kchunk,
                                                              double* __restrict__ part) {
+    chain_wait();
     __shared__ double As[TN_T][TN_T + 1];
     __shared__ double Bs[TN_T][TN_NARROW + 1];
     const int i0 = blockIdx.x * TN_T;
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(256) gemm_tn_narrow_kernel(const double* __res
 // is splits / 32 long; the partial sums are added in a fixed order.
 __global__ void __launch_bounds__(256) gemm_tn_reduce(const double* __restrict__ part, int splits, int m, int n,
                                                       double alpha, double beta, double* C, int64_t ldc) {
+    chain_wait();
     __shared__ double red[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int total = m * n;
@@ -165,6 +168,7 @@ __global__ void __launch_bounds__(256) gemm_nn_kernel(const double* __restrict__
                                                       const double* __restrict__ B, int64_t ldb,
                                                       double* C, int64_t ldc, int64_t K, int m,
                                                       int n, double alpha, double beta) {
+    chain_wait();
     __shared__ double Bs[NN_MB][NN_C];
     __shared__ double red[NN_G][NN_R][NN_C + 1];
     const int r = threadIdx.x % NN_R, g = threadIdx.x / NN_R;
@@ -207,6 +211,7 @@ __global__ void __launch_bounds__(256) gemm_nn_kernel(const double* __restrict__
 
 // ------------------------------ chol_rinv ---------------------------------
 __global__ void __launch_bounds__(256) chol_rinv_kernel(double* G, int n, double* Rinv, int* bad) {
+    chain_wait();
     __shared__ double s_d;
     __shared__ int s_bad;
     __shared__ double s_maxd;
@@ -281,6 +286,7 @@ __device__ inline double rsqrt_newton(double x) {
 }
 
 __global__ void __launch_bounds__(256) chol_rinv_smem_kernel(double* G, int n, double* Rinv, int* bad) {
+    chain_wait();
     extern __shared__ double sm[];
     double* L = sm;                       // n x n, column-major
     double* X = L + int64_t(n) * n;       // L^-1, column-major
@@ -379,15 +385,15 @@ cudaError_t launch_gemm_tn(const double* A, int64_t lda, const double* B, int64_
     const int64_t kchunk = ((K + splits - 1) / splits + TN_T - 1) / TN_T * TN_T;
     if (n <= TN_NARROW) {
         dim3 grid((m + TN_T - 1) / TN_T, 1, splits);
-        gemm_tn_narrow_kernel<<<grid, 256, 0, s>>>(A, lda, B, ldb, m, n, K, kchunk, scratch);
+        launch_chain(gemm_tn_narrow_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
     } else {
         dim3 grid((m + TN_T - 1) / TN_T, (n + TN_T - 1) / TN_T, splits);
-        gemm_tn_kernel<<<grid, 256, 0, s>>>(A, lda, B, ldb, m, n, K, kchunk, scratch);
+        launch_chain(gemm_tn_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int g = std::max(1, std::min(device_sm_count() * 8, (m * n + 31) / 32));
-    gemm_tn_reduce<<<g, 256, 0, s>>>(scratch, splits, m, n, alpha, beta, C, ldc);
+    launch_chain(gemm_tn_reduce, g, 256, 0, s, scratch, splits, m, n, alpha, beta, C, ldc);
     return cudaGetLastError();
 }
 
@@ -399,7 +405,7 @@ cudaError_t launch_gemm_nn(const double* A, int64_t lda, const double* B, int64_
     KL_RANGE(B, block_extent(m, n, ldb), double, "gemm_nn B");
     KL_RANGE(C, block_extent(K, n, ldc), double, "gemm_nn C");
     dim3 grid(unsigned((K + NN_R - 1) / NN_R), unsigned((n + NN_C - 1) / NN_C));
-    gemm_nn_kernel<<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, K, m, n, alpha, beta);
+    launch_chain(gemm_nn_kernel, grid, 256, 0, s, A, lda, B, ldb, C, ldc, K, m, n, alpha, beta);
     return cudaGetLastError();
 }
 
@@ -415,10 +421,10 @@ cudaError_t launch_chol_rinv(double* G, int n, double* Rinv, int* bad, cudaStrea
                                               int(chol_smem_bytes(kCholSmemN)));
         });
         if (attr_error != cudaSuccess) return attr_error;
-        chol_rinv_smem_kernel<<<1, 256, chol_smem_bytes(n), s>>>(G, n, Rinv, bad);
+        launch_chain(chol_rinv_smem_kernel, 1, 256, chol_smem_bytes(n), s, G, n, Rinv, bad);
         return cudaGetLastError();
     }
-    chol_rinv_kernel<<<1, 256, n * sizeof(double), s>>>(G, n, Rinv, bad);
+    launch_chain(chol_rinv_kernel, 1, 256, n * sizeof(double), s, G, n, Rinv, bad);
     return cudaGetLastError();
 }
 

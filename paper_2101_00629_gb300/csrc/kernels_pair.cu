@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
     int64_t T, const double* __restrict__ sx, const double* __restrict__ sy,
     const double* __restrict__ sz, int64_t S, const double* __restrict__ X, int64_t ldx, int k,
     int c0, double a, double* __restrict__ part, int64_t per_split) {
+    chain_wait();
     __shared__ double s_x[kSrc], s_y[kSrc], s_z[kSrc];
     __shared__ double s_v[kSrc][KB];
     const int64_t t = int64_t(blockIdx.x) * kTgt + threadIdx.x;
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     int64_t T, const double* __restrict__ sx, const double* __restrict__ sy,
     const double* __restrict__ sz, SrcGrid sg, const double* __restrict__ X, int64_t ldx, int k,
     int c0, double a, FxScale sc, double* __restrict__ part, int64_t per_split) {
+    chain_wait();
     constexpr int NG = KB > 8 ? 2 : 4;  // groups per stage
     constexpr int ST = 32 * NG;
     constexpr int Q = fx::Format<KIND>::kCoord, QA = fx::Format<KIND>::kArg;
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(kTgt) pair_f32_kernel(
     int64_t T, const float* __restrict__ sx, const float* __restrict__ sy,
     const float* __restrict__ sz, int64_t S, const double* __restrict__ X, int64_t ldx, int k,
     int c0, float a, float a2, double* __restrict__ part, int64_t per_split) {
+    chain_wait();
     __shared__ float4 s_c[kSrc];
     __shared__ __align__(16) float s_v[kSrc][KB];
     const int64_t t0 = int64_t(blockIdx.x) * (kTgt * R) + threadIdx.x;
@@ -411,6 +414,7 @@ __global__ void __launch_bounds__(32 * kRedSlices) pair_reduce_kernel(const doub
                                                                       int64_t T, int k, double sigma2,
                                                                       const double* __restrict__ post, double* Y,
                                                                       int64_t ldy) {
+    chain_wait();
     __shared__ double sh[kRedSlices][32];
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
     const int per = (splits + kRedSlices - 1) / kRedSlices;
@@ -442,7 +446,7 @@ cudaError_t run_pair_reduce(const double* part, int splits, int64_t T, int k, do
                             double* Y, int64_t ldy, cudaStream_t s) {
     const int64_t blocks = (T + 31) / 32 * k;
     const int g = int(std::min<int64_t>(blocks, int64_t(device_sm_count()) * 32));
-    pair_reduce_kernel<<<g < 1 ? 1 : g, 32 * kRedSlices, 0, s>>>(part, splits, T, k, sigma2, post, Y, ldy);
+    launch_chain(pair_reduce_kernel, g < 1 ? 1 : g, 32 * kRedSlices, 0, s, part, splits, T, k, sigma2, post, Y, ldy);
     return cudaGetLastError();
 }
 
@@ -480,11 +484,11 @@ void launch_f64(const PairArgs& a, int c0, int64_t per_split, cudaStream_t s) {
     const dim3 grid(unsigned((a.T + kTgt - 1) / kTgt), unsigned(a.splits));
     const int kc = a.k - c0;
     if (kc <= 8)
-        pair_f64_kernel<KIND, 8><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
+        launch_kernel(few_blocks(grid), pair_f64_kernel<KIND, 8>, grid, kTgt, 0, s, a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
     else if (kc <= 16)
-        pair_f64_kernel<KIND, 16><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
+        launch_kernel(few_blocks(grid), pair_f64_kernel<KIND, 16>, grid, kTgt, 0, s, a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
     else
-        pair_f64_kernel<KIND, 32><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
+        launch_kernel(few_blocks(grid), pair_f64_kernel<KIND, 32>, grid, kTgt, 0, s, a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, a.S, a.X, a.ldx, a.k, c0, a.ks.a, a.scratch, per_split);
 }
 
 // Blocks of the source grid: from one point, double the block along the
@@ -519,7 +523,7 @@ void launch_fx(const PairArgs& a, int c0, const FxScale& sc, const SrcGrid& sg, 
     const int64_t per_split = (sg.groups() + a.splits - 1) / a.splits;
     const dim3 grid(unsigned((a.T + kTgt - 1) / kTgt), unsigned(a.splits));
     auto go = [&](auto kb) {
-        pair_fx_kernel<KIND, decltype(kb)::value><<<grid, kTgt, 0, s>>>(a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, sg, a.X, a.ldx, a.k, c0, a.ks.a, sc, a.scratch, per_split);
+        launch_kernel(few_blocks(grid), pair_fx_kernel<KIND, decltype(kb)::value>, grid, kTgt, 0, s, a.tx, a.ty, a.tz, a.T, a.sx, a.sy, a.sz, sg, a.X, a.ldx, a.k, c0, a.ks.a, sc, a.scratch, per_split);
     };
     if (kc <= 1) go(std::integral_constant<int, 1>{});
     else if (kc <= 2) go(std::integral_constant<int, 2>{});
@@ -563,7 +567,7 @@ cudaError_t launch_kind(const PairArgs& a, bool fp32, cudaStream_t s) {
             auto go = [&](auto kb, auto r) {
                 constexpr int KB = decltype(kb)::value, R = decltype(r)::value;
                 const dim3 grid(unsigned((a.T + kTgt * R - 1) / (kTgt * R)), unsigned(a.splits));
-                pair_f32_kernel<KIND, KB, R><<<grid, kTgt, 0, s>>>(a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
+                launch_kernel(few_blocks(grid), pair_f32_kernel<KIND, KB, R>, grid, kTgt, 0, s, a.tx32, a.ty32, a.tz32, a.T, a.sx32, a.sy32, a.sz32, a.S, a.X, a.ldx, a.k, c0, fa, fa2, a.scratch, per_split);
             };
             using I1 = std::integral_constant<int, 1>;
             using I2 = std::integral_constant<int, 2>;

@@ -59,6 +59,7 @@ __global__ void tensor_points_kernel(int geometry, double g0, double g1, double 
                                      const double* __restrict__ w1, const double* __restrict__ w2,
                                      const double* __restrict__ w3, double jac_power, double* out_x,
                                      double* out_y, double* out_z, double* out_w) {
+    chain_wait();
     const int64_t n = int64_t(n1) * n2 * n3;
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
          i += int64_t(gridDim.x) * blockDim.x) {
@@ -123,6 +124,7 @@ __global__ void modeprod_kernel(const double* __restrict__ A, int m, int n,
                                 const double* __restrict__ X, int64_t ldx, double* __restrict__ Y,
                                 int64_t ldy, I a, I b, int k, const double* __restrict__ post,
                                 const double* __restrict__ pre) {
+    chain_wait();
     const I per_col = a * I(m) * b;
     for (int64_t c = blockIdx.y; c < k; c += gridDim.y) {
     for (I r = I(blockIdx.x) * blockDim.x + threadIdx.x; r < per_col; r += I(gridDim.x) * blockDim.x) {
@@ -166,6 +168,7 @@ __global__ void modeprod_band_kernel(const double* __restrict__ V, const int* __
                                      int n, const double* __restrict__ X, int64_t ldx, double* __restrict__ Y,
                                      int64_t ldy, I a, I b, int k, const double* __restrict__ post,
                                      const double* __restrict__ pre) {
+    chain_wait();
     const I per_col = a * I(m) * b;
     for (int64_t c = blockIdx.y; c < k; c += gridDim.y) {
     for (I r = I(blockIdx.x) * blockDim.x + threadIdx.x; r < per_col; r += I(gridDim.x) * blockDim.x) {
@@ -201,6 +204,7 @@ __device__ inline unsigned long long splitmix64(unsigned long long x) {
 // Box-Muller (one output per counter).
 __global__ void randn_kernel(double* X, int64_t ldx, int64_t K, int n, unsigned long long seed,
                              unsigned long long offset) {
+    chain_wait();
     const int64_t total = K * n;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
          t += int64_t(gridDim.x) * blockDim.x) {
@@ -216,6 +220,7 @@ __global__ void randn_kernel(double* X, int64_t ldx, int64_t K, int n, unsigned 
 
 __global__ void scale_cols_kernel(double* X, int64_t ldx, int64_t K, int n,
                                   const double* __restrict__ s, int invert) {
+    chain_wait();
     const int64_t total = K * n;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
          t += int64_t(gridDim.x) * blockDim.x) {
@@ -227,6 +232,7 @@ __global__ void scale_cols_kernel(double* X, int64_t ldx, int64_t K, int n,
 
 // X(i, j) *= scale[i] (K x n block, column-major).
 __global__ void scale_rows_kernel(double* X, int64_t ldx, int64_t K, int n, const double* __restrict__ scale) {
+    chain_wait();
     for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < K * n; e += int64_t(gridDim.x) * blockDim.x) {
         const int64_t i = e % K, j = e / K;
         X[i + j * ldx] *= scale[i];
@@ -237,6 +243,7 @@ __global__ void scale_rows_kernel(double* X, int64_t ldx, int64_t K, int n, cons
 // scale_out = scale / W.
 __global__ void rational_scales_kernel(double* w_inv, const double* __restrict__ scale,
                                        double* __restrict__ scale_out, int64_t n) {
+    chain_wait();
     for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
         const double inv = 1.0 / w_inv[i];
         w_inv[i] = inv;
@@ -246,6 +253,7 @@ __global__ void rational_scales_kernel(double* w_inv, const double* __restrict__
 
 __global__ void copy_block_kernel(const double* __restrict__ X, int64_t ldx, double* Y,
                                   int64_t ldy, int64_t K, int n) {
+    chain_wait();
     const int64_t total = K * n;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
          t += int64_t(gridDim.x) * blockDim.x) {
@@ -272,6 +280,7 @@ __device__ inline double block_sum(double v, double* sh) {
 // One block per column: out[c] = sqrt(sum_i w_i X_ic^2) (w may be NULL).
 __global__ void weighted_norms_kernel(const double* __restrict__ X, int64_t ldx, int64_t K,
                                       const double* __restrict__ w, double* out) {
+    chain_wait();
     // four independent loads and partial sums per step: one dependent chain
     // of DRAM round trips per thread would be K / blockDim long
     __shared__ double sh[32];
@@ -301,6 +310,7 @@ __global__ void weighted_norms_kernel(const double* __restrict__ X, int64_t ldx,
 // One block per column: flip the sign so that the largest-magnitude entry is
 // positive (first index wins ties).
 __global__ void sign_fix_kernel(double* X, int64_t ldx, int64_t K) {
+    chain_wait();
     __shared__ double sv[kThreads];
     __shared__ int64_t si[kThreads];
     const int c = blockIdx.x;
@@ -336,6 +346,7 @@ __global__ void sign_fix_kernel(double* X, int64_t ldx, int64_t K) {
 __global__ void resid_norms_kernel(const double* __restrict__ Y, int64_t ldy,
                                    const double* __restrict__ AY, int64_t lday,
                                    const double* __restrict__ theta, int64_t K, double* out) {
+    chain_wait();
     // four independent loads and partial sums per step (see weighted_norms_kernel)
     __shared__ double sh[32];
     const int c = blockIdx.x;
@@ -381,7 +392,7 @@ cudaError_t launch_tensor_points(int geometry, const double* geo, const double* 
     KL_RANGE(out_y, n, double, "tensor_points y");
     KL_RANGE(out_z, n, double, "tensor_points z");
     KL_RANGE(out_w, n, double, "tensor_points w");
-    tensor_points_kernel<<<grid_for(n), kThreads, 0, s>>>(geometry, geo[0], geo[1], geo[2], t1, t2,
+    launch_chain(tensor_points_kernel, grid_for(n), kThreads, 0, s, geometry, geo[0], geo[1], geo[2], t1, t2,
                                                           t3, n1, n2, n3, w1, w2, w3, jac_power,
                                                           out_x, out_y, out_z, out_w);
     return cudaGetLastError();
@@ -399,10 +410,10 @@ cudaError_t launch_modeprod(const double* A, int m, int n, const double* X, int6
     KL_RANGE(pre, a * n * b, double, "modeprod pre");
     const int64_t per_col = a * m * b;
     if (per_col < (int64_t(1) << 31))
-        modeprod_kernel<uint32_t><<<grid_cols(per_col, k), kThreads, 0, s>>>(A, m, n, X, ldx, Y, ldy, uint32_t(a),
+        launch_chain(modeprod_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint32_t(a),
                                                                              uint32_t(b), k, post, pre);
     else
-        modeprod_kernel<uint64_t><<<grid_cols(per_col, k), kThreads, 0, s>>>(A, m, n, X, ldx, Y, ldy, uint64_t(a),
+        launch_chain(modeprod_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint64_t(a),
                                                                              uint64_t(b), k, post, pre);
     return cudaGetLastError();
 }
@@ -420,10 +431,10 @@ cudaError_t launch_modeprod_band(const Band& A, int m, int n, const double* X, i
     KL_RANGE(pre, a * n * b, double, "band modeprod pre");
     const int64_t per_col = a * m * b;
     if (per_col < (int64_t(1) << 31))
-        modeprod_band_kernel<uint32_t><<<grid_cols(per_col, k), kThreads, 0, s>>>(
+        launch_chain(modeprod_band_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, 
             A.vals, A.start, A.w, m, n, X, ldx, Y, ldy, uint32_t(a), uint32_t(b), k, post, pre);
     else
-        modeprod_band_kernel<uint64_t><<<grid_cols(per_col, k), kThreads, 0, s>>>(
+        launch_chain(modeprod_band_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, 
             A.vals, A.start, A.w, m, n, X, ldx, Y, ldy, uint64_t(a), uint64_t(b), k, post, pre);
     return cudaGetLastError();
 }
@@ -434,14 +445,14 @@ cudaError_t launch_rational_scales(double* w_inv, const double* scale, double* s
     KL_RANGE(w_inv, n, double, "rational w_inv");
     KL_RANGE(scale, n, double, "rational scale");
     KL_RANGE(scale_out, n, double, "rational scale_out");
-    rational_scales_kernel<<<grid_for(n), kThreads, 0, s>>>(w_inv, scale, scale_out, n);
+    launch_chain(rational_scales_kernel, grid_for(n), kThreads, 0, s, w_inv, scale, scale_out, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_randn(double* X, int64_t ldx, int64_t K, int n, unsigned long long seed,
                          unsigned long long offset, cudaStream_t s) {
     KL_RANGE(X, block_extent(K, n, ldx), double, "randn X");
-    randn_kernel<<<grid_for(K * n), kThreads, 0, s>>>(X, ldx, K, n, seed, offset);
+    launch_chain(randn_kernel, grid_for(K * n), kThreads, 0, s, X, ldx, K, n, seed, offset);
     return cudaGetLastError();
 }
 
@@ -449,7 +460,7 @@ cudaError_t launch_scale_cols(double* X, int64_t ldx, int64_t K, int n, const do
                               int invert, cudaStream_t s) {
     KL_RANGE(X, block_extent(K, n, ldx), double, "scale_cols X");
     KL_RANGE(scale, n, double, "scale_cols scale");
-    scale_cols_kernel<<<grid_for(K * n), kThreads, 0, s>>>(X, ldx, K, n, scale, invert);
+    launch_chain(scale_cols_kernel, grid_for(K * n), kThreads, 0, s, X, ldx, K, n, scale, invert);
     return cudaGetLastError();
 }
 
@@ -457,7 +468,7 @@ cudaError_t launch_scale_rows(double* X, int64_t ldx, int64_t K, int n, const do
     if (K * n == 0) return cudaSuccess;
     KL_RANGE(X, block_extent(K, n, ldx), double, "scale_rows X");
     KL_RANGE(scale, K, double, "scale_rows scale");
-    scale_rows_kernel<<<grid_for(K * n), kThreads, 0, s>>>(X, ldx, K, n, scale);
+    launch_chain(scale_rows_kernel, grid_for(K * n), kThreads, 0, s, X, ldx, K, n, scale);
     return cudaGetLastError();
 }
 
@@ -466,7 +477,7 @@ cudaError_t launch_copy_block(const double* X, int64_t ldx, double* Y, int64_t l
     if (K * n == 0) return cudaSuccess;
     KL_RANGE(X, block_extent(K, n, ldx), double, "copy_block X");
     KL_RANGE(Y, block_extent(K, n, ldy), double, "copy_block Y");
-    copy_block_kernel<<<grid_for(K * n), kThreads, 0, s>>>(X, ldx, Y, ldy, K, n);
+    launch_chain(copy_block_kernel, grid_for(K * n), kThreads, 0, s, X, ldx, Y, ldy, K, n);
     return cudaGetLastError();
 }
 
@@ -474,7 +485,7 @@ cudaError_t launch_col_norms(const double* X, int64_t ldx, int64_t K, int n, dou
                              cudaStream_t s) {
     KL_RANGE(X, block_extent(K, n, ldx), double, "col_norms X");
     KL_RANGE(out, n, double, "col_norms out");
-    weighted_norms_kernel<<<n, kThreads, 0, s>>>(X, ldx, K, nullptr, out);
+    launch_chain(weighted_norms_kernel, n, kThreads, 0, s, X, ldx, K, nullptr, out);
     return cudaGetLastError();
 }
 
@@ -483,13 +494,13 @@ cudaError_t launch_weighted_norms(const double* X, int64_t ldx, int64_t K, int n
     KL_RANGE(X, block_extent(K, n, ldx), double, "weighted_norms X");
     KL_RANGE(w, K, double, "weighted_norms w");
     KL_RANGE(out, n, double, "weighted_norms out");
-    weighted_norms_kernel<<<n, kThreads, 0, s>>>(X, ldx, K, w, out);
+    launch_chain(weighted_norms_kernel, n, kThreads, 0, s, X, ldx, K, w, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sign_fix(double* X, int64_t ldx, int64_t K, int n, cudaStream_t s) {
     KL_RANGE(X, block_extent(K, n, ldx), double, "sign_fix X");
-    sign_fix_kernel<<<n, kThreads, 0, s>>>(X, ldx, K);
+    launch_chain(sign_fix_kernel, n, kThreads, 0, s, X, ldx, K);
     return cudaGetLastError();
 }
 
@@ -500,7 +511,7 @@ cudaError_t launch_resid_norms(const double* Y, int64_t ldy, const double* AY, i
     KL_RANGE(AY, block_extent(K, n, lday), double, "resid_norms AY");
     KL_RANGE(theta, n, double, "resid_norms theta");
     KL_RANGE(out, n, double, "resid_norms out");
-    resid_norms_kernel<<<n, kThreads, 0, s>>>(Y, ldy, AY, lday, theta, K, out);
+    launch_chain(resid_norms_kernel, n, kThreads, 0, s, Y, ldy, AY, lday, theta, K, out);
     return cudaGetLastError();
 }
 

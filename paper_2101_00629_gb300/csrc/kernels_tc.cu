@@ -404,6 +404,7 @@ __global__ void tc_convert_kernel(const double* __restrict__ X, int64_t ldx, int
                                   int np, int kchunk, bool tf32, float cscale, const float* __restrict__ sx,
                                   const float* __restrict__ sy, const float* __restrict__ sz,
                                   uint8_t* __restrict__ img, int64_t nchunks) {
+    chain_wait();
     const int esize = tf32 ? 4 : 2;
     const int64_t img_bytes = int64_t(np) * kchunk * esize;  // one of hi / lo
     const int64_t rec_bytes = 2 * img_bytes + 12 * int64_t(kchunk);
@@ -543,6 +544,7 @@ constexpr uint32_t kSymTgtGroupStride = 128;    // along K (targets)
 template <int KIND, bool TF32, int NP, bool SYM>
 __global__ void __launch_bounds__(kThreads, 2)
 pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
+    chain_wait();
     static_assert(!SYM || (!TF32 && NP == 16), "symmetric mode: split BF16, N = 16");
     const int64_t nunits = batch.nunits;
     const long long wlim = batch.wait_limit > 0 ? batch.wait_limit : kWaitLimit;
@@ -1012,7 +1014,7 @@ cudaError_t launch_batch_np(const TcBatch& b, int sm_count, int* err, cudaStream
     std::call_once(once, [&] { attr_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (attr_error != cudaSuccess) return attr_error;
     const int64_t grid = std::min<int64_t>(b.nunits, 2LL * sm_count);
-    kern<<<unsigned(grid), kThreads, smem, s>>>(b, err);
+    launch_kernel(b.chained != 0, kern, unsigned(grid), kThreads, smem, s, b, err);
     return cudaGetLastError();
 }
 
@@ -1065,6 +1067,7 @@ constexpr int kRedSplit = 8;
 __global__ void __launch_bounds__(32 * kRedSplit)
 tc_reduce_kernel(const float2* __restrict__ part, int splits, int64_t T, int k, double sigma2,
                  const double* __restrict__ post, double* __restrict__ Y, int64_t ldy) {
+    chain_wait();
     __shared__ float2 sh[kRedSplit][32];
     const int64_t tblocks = (T + 31) / 32;
     const int y = threadIdx.y;
@@ -1126,6 +1129,7 @@ tc_sym_reduce_kernel(const float2* __restrict__ part1, const float* __restrict__
                      const int2* __restrict__ tab, int64_t nchunks, int64_t T, int k, int tile0, int tile1,
                      int64_t unit_begin, int first, float2* __restrict__ acc, double sigma2,
                      const double* __restrict__ post, double* __restrict__ Y, int64_t ldy) {
+    chain_wait();
     __shared__ float4 sh[kSymRedThreads][2];
     const int kstride = (k + 7) & ~7;
     const int ng = kstride / 4;   // 16-byte column groups per row
@@ -1285,7 +1289,7 @@ cudaError_t tc_prepare(const TcArgs& a, cudaStream_t s, TcInstance* out, int* n,
         uint8_t* img = reinterpret_cast<uint8_t*>(a.scratch + blk * p.img_blk_doubles);
         const int64_t total = p.nchunks * p.kchunk * p.np_max;
         const int g = int(std::min<int64_t>((total + 255) / 256, int64_t(a.sm_count) * 64));
-        tc_convert_kernel<<<g, 256, 0, s>>>(a.X, a.ldx, a.S, c0, kc, p.np_max, p.kchunk, a.tf32, cscale, a.sx,
+        launch_chain(tc_convert_kernel, g, 256, 0, s, a.X, a.ldx, a.S, c0, kc, p.np_max, p.kchunk, a.tf32, cscale, a.sx,
                                             a.sy, a.sz, img, p.nchunks);
         ++*launched;
         cudaError_t e = cudaGetLastError();
@@ -1348,7 +1352,7 @@ cudaError_t tc_launch_batch(TcBatch& b, bool tf32, int np, int sm_count, int* er
                 : launch_batch_prec<false>(b, np, false, sm_count, err, s);
 }
 
-cudaError_t tc_finish(const TcArgs& a, cudaStream_t s, int* launched) {
+cudaError_t tc_finish(const TcArgs& a, cudaStream_t s, int* launched, bool chained) {
     const TcPlan p = plan(a.T, a.S, a.k, a.sm_count, a.tf32);
     const float2* part = reinterpret_cast<const float2*>(a.scratch + p.img_doubles + p.src_doubles);
     KL_RANGE(part, p.part_doubles, float2, "tc_reduce partial sums");
@@ -1356,7 +1360,7 @@ cudaError_t tc_finish(const TcArgs& a, cudaStream_t s, int* launched) {
     KL_RANGE(a.post, a.T, double, "tc_reduce post");
     const int64_t nblk = (a.T + 31) / 32 * a.k;
     const int g = int(std::max<int64_t>(1, std::min<int64_t>(nblk, int64_t(a.sm_count) * 16)));
-    tc_reduce_kernel<<<g, dim3(32, kRedSplit), 0, s>>>(part, p.splits, a.T, a.k, a.ks.sigma2, a.post, a.Y, a.ldy);
+    launch_kernel(chained, tc_reduce_kernel, g, dim3(32, kRedSplit), 0, s, part, p.splits, a.T, a.k, a.ks.sigma2, a.post, a.Y, a.ldy);
     ++*launched;
     return cudaGetLastError();
 }
@@ -1453,7 +1457,7 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
     {
         const int64_t total = p.nchunks * 64 * 16;
         const int g = int(std::min<int64_t>((total + 255) / 256, int64_t(a.sm_count) * 64));
-        tc_convert_kernel<<<g, 256, 0, s>>>(a.X, a.ldx, a.S, 0, a.k, 16, 64, false, cscale, a.sx, a.sy, a.sz, img,
+        launch_chain(tc_convert_kernel, g, 256, 0, s, a.X, a.ldx, a.S, 0, a.k, 16, 64, false, cscale, a.sx, a.sy, a.sz, img,
                                             p.nchunks);
         ++*launched;
         cudaError_t e = cudaGetLastError();
@@ -1465,6 +1469,7 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
         TcBatch batch;
         batch.ninst = 1;
         batch.wait_limit = a.wait_limit;
+        batch.chained = 1;
         TcInstance& I = batch.inst[0];
         I.tx = a.tx;
         I.ty = a.ty;
@@ -1509,7 +1514,7 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
         if (e != cudaSuccess) return e;
         // one block per chunk of the band's points and the later ones
         const int g = int(std::max<int64_t>(1, p.nchunks - 2 * int64_t(tile0)));
-        tc_sym_reduce_kernel<<<g, kSymRedThreads, 0, s>>>(part1, part2, tab, p.nchunks, a.T, a.k, tile0, tile1,
+        launch_chain(tc_sym_reduce_kernel, g, kSymRedThreads, 0, s, part1, part2, tab, p.nchunks, a.T, a.k, tile0, tile1,
                                                I.sym_unit_begin, b == 0, acc, a.ks.sigma2, a.post,
                                                a.Y, a.ldy);
         ++*launched;
@@ -1523,13 +1528,14 @@ cudaError_t launch_pair_tc(const TcArgs& a, cudaStream_t s, int* launched) {
     *launched = 0;
     TcBatch b;
     b.wait_limit = a.wait_limit;
+    b.chained = 1;
     int np = 16;
     cudaError_t e = tc_prepare(a, s, b.inst, &b.ninst, &np, launched);
     if (e != cudaSuccess) return e;
     e = tc_launch_batch(b, a.tf32, np, a.grid_sms > 0 ? a.grid_sms : a.sm_count, a.err, s);
     ++*launched;
     if (e != cudaSuccess) return e;
-    return tc_finish(a, s, launched);
+    return tc_finish(a, s, launched, true);
 }
 
 }  // namespace kl

@@ -67,6 +67,7 @@ struct TcBatch {
     int ninst;
     int64_t nunits;
     long long wait_limit;  // clock cycles of each pipeline wait (0: about a second)
+    int chained;           // launched behind its own conversion on the same stream
 };
 
 // Phase 1 of a pairwise product: conversion kernels on stream s and the
@@ -77,7 +78,7 @@ cudaError_t tc_prepare(const TcArgs& a, cudaStream_t s, TcInstance* out, int* n,
 // units assigned contiguously in order; err: device word set on a timeout.
 cudaError_t tc_launch_batch(TcBatch& b, bool tf32, int np, int sm_count, int* err, cudaStream_t s);
 // Phase 3: reduction of the partial sums into Y on stream s.
-cudaError_t tc_finish(const TcArgs& a, cudaStream_t s, int* launched);
+cudaError_t tc_finish(const TcArgs& a, cudaStream_t s, int* launched, bool chained);
 // Scratch needed by launch_pair_tc for T targets and any block of at most k
 // vectors (doubles).
 int64_t tc_scratch_doubles(int64_t T, int64_t S, int k, int sm_count);

@@ -157,6 +157,7 @@ void Batcher::loop() {
             TcBatch b;
             b.ninst = 0;
             b.wait_limit = 0;
+            b.chained = 0;  // waits for events of other streams
             ErrTargets et;
             et.n = 0;
             cudaError_t err = cudaSuccess;
