@@ -132,6 +132,84 @@ void domain_extent(const kl_params& p, double* e) {
 // Precisions whose pairwise product runs on the CUDA cores.
 bool cuda_cores(int precision) { return precision == KL_FP64 || precision == KL_FP32; }
 
+// Factors of the direction's Z as LineSolve stores them (lo, up, fs, bs in one
+// vector); empty if the matrix does not have the band or the factorisation
+// does not reproduce it.
+std::vector<double> pack_lines(int n, int p, const std::vector<double>& lo, const std::vector<double>& up,
+                               const std::vector<double>& fs, const std::vector<double>& bs) {
+    std::vector<double> v;
+    v.reserve(size_t(n) * (2 * p + 2));
+    for (const std::vector<double>* x : {&lo, &up, &fs, &bs}) v.insert(v.end(), x->begin(), x->end());
+    return v;
+}
+
+// Z = L L^T: forward L^-1, backward L^-T.
+std::vector<double> cholesky_lines(const Mat& L, int p) {
+    const int n = L.rows;
+    std::vector<double> lo(size_t(n) * p, 0.0), up(size_t(n) * p, 0.0), inv(n);
+    for (int i = 0; i < n; ++i) {
+        inv[i] = 1.0 / L(i, i);
+        for (int j = 0; j < i; ++j)
+            if (i - j > p && L(i, j) != 0.0) return {};
+    }
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < p; ++j) {
+            if (i - 1 - j >= 0) lo[size_t(i) * p + j] = L(i, i - 1 - j) * inv[i];
+            if (i + 1 + j < n) up[size_t(i) * p + j] = L(i + 1 + j, i) * inv[i];
+        }
+    return pack_lines(n, p, lo, up, inv, inv);
+}
+
+// Z = L U without pivoting: forward L^-1 (unit diagonal), backward U^-1.
+std::vector<double> lu_lines(const Mat& Z, int p) {
+    const int n = Z.rows;
+    double top = 0.0;
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) {
+            top = std::max(top, std::fabs(Z(i, j)));
+            if ((i - j > p || j - i > p) && Z(i, j) != 0.0) return {};
+        }
+    Mat F = Z;
+    for (int c = 0; c < n; ++c) {
+        if (!(std::fabs(F(c, c)) > 1e-8 * top)) return {};
+        for (int i = c + 1; i < std::min(n, c + p + 1); ++i) {
+            F(i, c) /= F(c, c);
+            if (std::fabs(F(i, c)) > 1e3) return {};
+            for (int j = c + 1; j < std::min(n, c + p + 1); ++j) F(i, j) -= F(i, c) * F(c, j);
+        }
+    }
+    std::vector<double> lo(size_t(n) * p, 0.0), up(size_t(n) * p, 0.0), one(n, 1.0), inv(n);
+    for (int i = 0; i < n; ++i) {
+        inv[i] = 1.0 / F(i, i);
+        for (int j = 0; j < p; ++j) {
+            if (i - 1 - j >= 0) lo[size_t(i) * p + j] = F(i, i - 1 - j);
+            if (i + 1 + j < n) up[size_t(i) * p + j] = F(i, i + 1 + j) * inv[i];
+        }
+        for (int j = 0; j < n; ++j) {  // L U = Z to rounding
+            double s = 0.0;
+            for (int l = std::max(0, i - p); l <= std::min(i, j); ++l) s += (l == i ? 1.0 : F(i, l)) * (j >= l && j - l <= p ? F(l, j) : 0.0);
+            if (std::fabs(s - Z(i, j)) > 1e-14 * top) return {};
+        }
+    }
+    return pack_lines(n, p, lo, up, one, inv);
+}
+
+// FMAs per column that one application of A' saves with the banded tables F,
+// F^T in place of the dense P = F L^-T and P^T (the solves not counted); 0 if a
+// table of a direction is dense.
+double split_saving(const kl_solver* h) {
+    double saved = 0.0, in = 1.0, out = 1.0;
+    for (int d = 0; d < 3; ++d) in *= h->N1[d], out *= h->Ns1[d];
+    double mid_pre = in, mid_post = out;
+    for (int d = 0; d < h->prm.dim; ++d) {
+        if (!h->bF[d].vals || !h->bFT[d].vals) return 0.0;
+        mid_pre *= double(h->Ns1[d]) / h->N1[d];
+        mid_post *= double(h->N1[d]) / h->Ns1[d];
+        saved += mid_pre * (h->N1[d] - h->bF[d].w) + mid_post * (h->Ns1[d] - h->bFT[d].w);
+    }
+    return saved;
+}
+
 template <class T>
 cudaError_t dalloc(kl_solver* h, T** p, int64_t count) {
     *p = nullptr;
@@ -154,23 +232,22 @@ int ensure_workspace(kl_solver* h, int k) {
     cudaError_t e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "workspace sync");
     clear_graphs(h);
-    for (int i = 0; i < 3; ++i) {
-        if (h->ws[i]) h->dev_bytes -= std::max(h->S, h->T) * int64_t(h->k_cap) * int64_t(sizeof(double));
-        dfree(h->ws[i]);
-        h->ws[i] = nullptr;
-    }
-    if (h->pair_scratch) h->dev_bytes -= h->pair_scratch_len * int64_t(sizeof(double));
-    dfree(h->pair_scratch);
-    h->pair_scratch = nullptr;
+    dfree(h->work);
+    h->dev_bytes -= h->work_len * int64_t(sizeof(double));
+    h->work = nullptr;
+    h->work_len = 0;
     h->k_cap = 0;
-    const int64_t big = std::max(h->S, h->T) * int64_t(k);
-    for (int i = 0; i < 3; ++i)
-        if ((e = dalloc(h, &h->ws[i], big)) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
+    // one allocation for the three operator blocks and the pairwise scratch:
+    // each of them costs tens of microseconds of handle creation
+    const int64_t big = (std::max(h->S, h->T) * int64_t(k) + 31) / 32 * 32;
     h->pair_splits = pair_choose_splits(h->T, h->S, h->sm_count, cuda_cores(h->prm.precision));
-    h->pair_scratch_len = std::max<int64_t>(pair_scratch_doubles(h->T, k, h->pair_splits),
-                                            tc_scratch_doubles(h->T, h->S, k, h->sm_count));
-    if ((e = dalloc(h, &h->pair_scratch, h->pair_scratch_len)) != cudaSuccess)
-        return cuda_fail(h, e, "pair scratch alloc");
+    const int64_t scratch = std::max<int64_t>(pair_scratch_doubles(h->T, k, h->pair_splits),
+                                              tc_scratch_doubles(h->T, h->S, k, h->sm_count));
+    if ((e = dalloc(h, &h->work, 3 * big + scratch)) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
+    h->work_len = 3 * big + scratch;
+    for (int i = 0; i < 3; ++i) h->ws[i] = h->work + i * big;
+    h->pair_scratch = h->work + 3 * big;
+    h->pair_scratch_len = scratch;
     h->k_cap = k;
     return KL_OK;
 }
@@ -258,6 +335,52 @@ static int kron3_s(kl_solver* h, const double* const* Fd, const int* n_in, const
         ldc = ldo;
     }
     return KL_OK;
+}
+
+// Y = Z^-1 X (both sweeps), L^-1 X (forward) or L^-T X (backward) through the
+// banded factors, one direction after the other; X and Y may be the same
+// block.
+static int line_solve3(kl_solver* h, bool fwd, bool bwd, const double* X, int64_t ldx, double* Y, int64_t ldy, int k,
+                       const double* post = nullptr, const double* pre = nullptr) {
+    int64_t a = 1, b = h->N;
+    for (int d = 0; d < h->prm.dim; ++d) {
+        b /= h->N1[d];
+        cudaError_t e = launch_line_solve(h->line[d], fwd, bwd, d == 0 ? X : Y, d == 0 ? ldx : ldy, Y, ldy, a, b, k,
+                                          d == h->prm.dim - 1 ? post : nullptr, d == 0 ? pre : nullptr, h->stream);
+        ++h->launches;
+        if (e != cudaSuccess) return cuda_fail(h, e, "line solve");
+        a *= h->N1[d];
+    }
+    return KL_OK;
+}
+
+// Time (us) of `sweeps` banded sweeps per direction over k columns, without the
+// launches: FP64 throughput (0.5 FMA per ps), or the chain of one line, whose
+// step is p + 1 operations of 80 cycles (50 ns with the loads). Measured for p =
+// 2: 18^3 dofs, both sweeps, k = 1, 24 us for the three launches, 66 x 34 x 18,
+// k = 32, 71 us.
+static double line_solve_us(const kl_solver* h, int sweeps, int k) {
+    const int ops = sweeps * (h->prm.degree + 1);
+    double work = 0.0, chain = 0.0;
+    for (int d = 0; d < h->prm.dim; ++d) {
+        work += double(h->N) * k * ops;
+        chain += double(h->N1[d]) * ops;
+    }
+    return std::max(work / 0.5e6, chain * 0.05);
+}
+
+// Z^-1 by banded solves or by the dense inverses (n FMAs per point and
+// direction): 26^3 dofs, p = 2: k = 1 29 and 17 us, k = 32 34 and 90 us.
+static bool zinv_by_lines(const kl_solver* h, int k) {
+    const double dense = double(h->N) * k * (h->N1[0] + h->N1[1] + h->N1[2]) / 0.5e6;
+    return h->line_solves && dense > 1.2 * line_solve_us(h, 2, k);
+}
+
+// A' as the solves L^-T and L^-1 around the banded tables of A: where the FMAs
+// it saves outweigh the sweeps and six more launches (10 us). 18^3 dofs, 33^3
+// points, k = 8, break even; 66 x 34 x 18 dofs, k = 32, save 2 ms.
+static bool split_form(const kl_solver* h, int k) {
+    return h->split_saved * k / 0.5e6 > 1.2 * (2.0 * line_solve_us(h, 1, k) + 10.0);
 }
 
 static int pairwise(kl_solver* h, int precision, const double* U, double* W, int k,
@@ -376,6 +499,10 @@ static int apply_pre(kl_solver* h, int which, const double* X, int64_t ldx, int 
     const bool proj = gal && which == 1;
     const double* const* F = proj ? h->P : h->F;
     const double* post = h->rat_w ? h->rat_src_scale : h->src_scale;
+    if (proj && split_form(h, k)) {
+        if (int rc = line_solve3(h, false, true, X, ldx, h->ws[1], h->N, k); rc != KL_OK) return rc;
+        return kron3(h, h->F, h->N1, h->Ns1, h->ws[1], h->N, h->ws[0], h->S, k, post, 2, 1, nullptr, h->bF);
+    }
     return kron3(h, F, h->N1, h->Ns1, X, ldx, h->ws[0], h->S, k, post, 1, 2, h->rat_w, proj ? nullptr : h->bF);
 }
 
@@ -386,7 +513,13 @@ static int apply_post(kl_solver* h, int which, double* Y, int64_t ldy, int k) {
     const bool proj = gal && which == 1;
     const double* const* FT = proj ? h->PT : h->FT;
     double* W = h->ws[1];
+    if (proj && split_form(h, k)) {
+        if (int rc = kron3(h, h->FT, h->Ns1, h->N1, W, h->T, Y, ldy, k, nullptr, 0, 2, nullptr, h->bFT); rc != KL_OK)
+            return rc;
+        return line_solve3(h, true, false, Y, ldy, Y, ldy, k);
+    }
     if (gal) return kron3(h, FT, h->Ns1, h->N1, W, h->T, Y, ldy, k, nullptr, 0, 2, nullptr, proj ? nullptr : h->bFT);
+    if (which == 1 && zinv_by_lines(h, k)) return line_solve3(h, true, true, W, h->T, Y, ldy, k, h->rat_invw, h->rat_Wc);
     if (which == 1) return kron3(h, h->Zinv, h->N1, h->N1, W, h->T, Y, ldy, k, h->rat_invw, 0, 2, h->rat_Wc);
     cudaError_t e = launch_copy_block(W, h->T, Y, ldy, h->T, k, h->stream);
     ++h->launches;
@@ -491,12 +624,14 @@ int apply_operator(kl_solver* h, int which, int precision, const double* X, int6
 // Z^-1 (Kronecker LU solves, Sec. 3.2); with non-tensor NURBS weights
 // Z = diag(1 / W(x_i)) B diag(w), so Z^-1 = diag(1 / w) B^-1 diag(W(x_i)).
 int apply_zinv(kl_solver* h, const double* X, int64_t ldx, double* Y, int64_t ldy, int k) {
+    if (zinv_by_lines(h, k)) return line_solve3(h, true, true, X, ldx, Y, ldy, k, h->rat_invw, h->rat_Wc);
     return kron3(h, h->Zinv, h->N1, h->N1, X, ldx, Y, ldy, k, h->rat_invw, 0, 1, h->rat_Wc);
 }
 
 int back_transform(kl_solver* h, const double* Yv, int64_t ldy, double* V, int64_t ldv, int k) {
     if (galerkin_form(h->prm.method))
-        return kron3(h, h->LinvT, h->N1, h->N1, Yv, ldy, V, ldv, k, nullptr, 0, 1);
+        return zinv_by_lines(h, k) ? line_solve3(h, false, true, Yv, ldy, V, ldv, k)
+                              : kron3(h, h->LinvT, h->N1, h->N1, Yv, ldy, V, ldv, k, nullptr, 0, 1);
     cudaError_t e = launch_copy_block(Yv, ldy, V, ldv, h->N, k, h->stream);
     ++h->launches;
     return e == cudaSuccess ? KL_OK : cuda_fail(h, e, "copy");
@@ -768,7 +903,21 @@ int kl_create(const kl_params* params, void* stream, kl_solver** out) {
                 pend.push_back(p);
             }
         }
-        if (!pend.empty()) {
+        // banded factors of Z per direction: Cholesky (Galerkin, A' needs its
+        // two triangles) or LU without pivoting (collocation at the Greville
+        // points: totally positive, so no pivoting is needed; checked)
+        size_t line_at[3] = {0, 0, 0};
+        for (int d = 0; d < p.dim; ++d) {
+            const std::vector<double> f = gal ? cholesky_lines(dir[d].L, p.degree) : lu_lines(dir[d].Zc, p.degree);
+            if (f.empty() || dir[d].N > kLineMaxN) continue;
+            h->line[d].n = dir[d].N;
+            h->line[d].p = p.degree;
+            line_at[d] = bv.size();
+            bv.insert(bv.end(), f.begin(), f.end());
+            while (bv.size() % 4) bv.push_back(0.0);
+        }
+        if (!bv.empty()) {
+            if (bs.empty()) bs.push_back(0);
             if ((e = dalloc(h, &h->d_band_vals, int64_t(bv.size()))) != cudaSuccess)
                 return bail(cuda_fail(h, e, "band alloc"));
             if ((e = device_alloc((void**)&h->d_band_start, bs.size() * sizeof(int))) != cudaSuccess)
@@ -787,6 +936,19 @@ int kl_create(const kl_params* params, void* stream, kl_solver** out) {
                 p.dst->start = h->d_band_start + p.s0;
                 p.dst->w = p.w;
             }
+            int have = 0;
+            for (int d = 0; d < p.dim; ++d) {
+                LineSolve& t = h->line[d];
+                if (t.p == 0) continue;
+                ++have;
+                const int64_t np = int64_t(t.n) * t.p;
+                t.lo = h->d_band_vals + line_at[d];
+                t.up = t.lo + np;
+                t.fs = t.up + np;
+                t.bs = t.fs + t.n;
+            }
+            h->line_solves = have == p.dim;
+            h->split_saved = gal && have == p.dim ? split_saving(h) : 0.0;
         }
     }
     for (int d = 0; d < 3; ++d) {
@@ -1022,6 +1184,7 @@ int kl_estimate_bytes(const kl_params* params, int M, int64_t* bytes) {
         add(ns);
         add(ns);
         add(int64_t(q.ne) * q.N);
+        add(int64_t(q.N) * (2 * p.degree + 2));  // banded factors of Z
         add(q.ne);
     }
     const int64_t S = Ns, T = gal ? S : N;
@@ -1059,8 +1222,7 @@ int kl_destroy(kl_solver* h) {
     dfree(h->d_rat);
     dfree(h->d_band_vals);
     dfree(h->d_band_start);
-    for (int i = 0; i < 3; ++i) dfree(h->ws[i]);
-    dfree(h->pair_scratch);
+    dfree(h->work);
     dfree(h->sym_scratch);
     delete h->sym_plan;
     dfree(h->eig_ws);

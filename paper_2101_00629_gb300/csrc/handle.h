@@ -58,6 +58,12 @@ struct kl_solver {
     kl::Band bF[3], bFT[3], bE[3];
     double* d_band_vals = nullptr;
     int* d_band_start = nullptr;
+    // banded factors of Z per direction (stored with the band tables), whether
+    // every direction has them, and the FMAs per column that A' saves with
+    // banded tables between solves (0: not all of them are banded)
+    kl::LineSolve line[3];
+    bool line_solves = false;
+    double split_saved = 0.0;
     const double* xe[3] = {};     // those Gauss points (parameters)
     int Ne1[3] = {1, 1, 1};       // Gauss points per direction (sampling grid)
 
@@ -84,6 +90,8 @@ struct kl_solver {
 
     // workspaces for operator applications (k_cap vectors)
     int k_cap = 0;
+    double* work = nullptr;  // one allocation of work_len doubles: ws, pair_scratch
+    int64_t work_len = 0;
     double* ws[3] = {nullptr, nullptr, nullptr};
     double* pair_scratch = nullptr;
     int64_t pair_scratch_len = 0;

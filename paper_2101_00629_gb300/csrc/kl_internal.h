@@ -46,6 +46,7 @@ struct Dir1D {
     Mat P;                      // B~^-T M L^-T        (Nt x N)
     Mat LinvT;                  // L^-T                (N x N)
     Mat Zinv_gal;               // Z^-1 = L^-T L^-1    (N x N)
+    Mat L;                      // Z = L L^T           (N x N)
     // Collocation
     int nq = 1;                 // quadrature points of this direction
     std::vector<double> xq, wq; // Gauss points / weights (nq)
@@ -59,6 +60,7 @@ struct Dir1D {
     std::vector<double> we;     // their Gauss weights (ne)
     Mat E;                      // trial basis at them (ne x N)
     Mat Zinv_col;               // (R_j(xc_i))^-1      (N x N)
+    Mat Zc;                     // R_j(xc_i)           (N x N)
 };
 
 // Both Galerkin forms (IBQ and standard quadrature): the trial space
@@ -184,6 +186,22 @@ cudaError_t launch_modeprod_band(const Band& A, int m, int n, const double* X, i
 cudaError_t launch_modeprod(const double* A, int m, int n, const double* X, int64_t ldx, double* Y,
                             int64_t ldy, int64_t a, int64_t b, int k, const double* post,
                             const double* pre, cudaStream_t s);
+// Banded triangular factors of an n x n matrix, applied along one direction:
+// forward  z_i = fs[i] x_i - sum_j lo[i p + j] z_(i-1-j)
+// backward y_i = bs[i] z_i - sum_j up[i p + j] y_(i+1+j)
+// (coefficients beyond the matrix are zero).
+struct LineSolve {
+    const double *lo = nullptr, *up = nullptr, *fs = nullptr, *bs = nullptr;
+    int n = 0, p = 0;  // p = 0: no factors (dense products instead)
+};
+constexpr int kLineMaxN = 552;  // 32 lines of a block and the coefficients in shared memory
+// Y = solve(X) along the direction of length t.n with `a` points of earlier
+// and b of later directions; the forward and/or the backward sweep. Optional
+// scalings of the input (pre) and output (post) points. X and Y may be the
+// same block.
+cudaError_t launch_line_solve(const LineSolve& t, bool forward, bool backward, const double* X, int64_t ldx,
+                              double* Y, int64_t ldy, int64_t a, int64_t b, int k, const double* post,
+                              const double* pre, cudaStream_t s);
 // w_inv <- 1 / w_inv (W at the Gauss points), scale_out = scale * (1 / W).
 cudaError_t launch_rational_scales(double* w_inv, const double* scale, double* scale_out, int64_t n,
                                    cudaStream_t s);

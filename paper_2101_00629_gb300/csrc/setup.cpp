@@ -345,6 +345,7 @@ std::string setup_direction(Dir1D& d, bool present, int nel, int p, int interp_c
         Mat L = Z;
         if (!cholesky(L)) return "1D mass matrix not positive definite";
         const Mat Linv = lower_inverse(L);
+        d.L = L;
         d.LinvT = transpose(Linv);
         d.Zinv_gal = matmul(d.LinvT, Linv);
         const Mat Bt = basis_matrix(Ut, d.xg, &xg_left);  // Bt(a, j) = B~_j(x~_a)
@@ -369,6 +370,7 @@ std::string setup_direction(Dir1D& d, bool present, int nel, int p, int interp_c
         d.R = rational_rows(BU, w);
         const Mat Zc = rational_rows(Bc, w);
         if (!lu_solve(Zc, identity(d.N), d.Zinv_col)) return "1D collocation matrix singular";
+        d.Zc = Zc;
     }
     d.ne = int(xq.size());
     d.xe = xq;
