@@ -550,7 +550,6 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
     const long long wlim = batch.wait_limit > 0 ? batch.wait_limit : kWaitLimit;
     constexpr int ESIZE = TF32 ? 4 : 2;
     constexpr int KC = TF32 ? 32 : 64;                  // sources per chunk (32 TMEM columns)
-    constexpr int SW = KC / 2;                          // sources of each warpgroup
     constexpr int IMG = NP * KC * ESIZE;                // bytes of one of hi / lo
     constexpr int STAGE_BYTES = 2 * IMG + KC * 12;      // hi, lo, coordinates x[KC] y[KC] z[KC]
     constexpr int SSTAGES = SYM ? kSymRecStages : smem_stages(STAGE_BYTES);  // shared-memory ring (>= kStages)
@@ -587,7 +586,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
             mbar_init(&sempty_bar[s], 1);
         }
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&full_bar[s], 256);  // both warpgroups write half of every tile
+            mbar_init(&full_bar[s], 128);  // the warpgroup that writes the tile
             mbar_init(&tfree_bar[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -599,7 +598,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&d2full_bar[b], 1);
-            mbar_init(&d2free_bar[b], 256);
+            mbar_init(&d2free_bar[b], 128);  // the warpgroup that drains the product
         }
         mbar_init(&drain_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -616,15 +615,14 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
     const uint32_t tmem = tmem_slot;
 
     if (warp < 8) {
-        // ---------------- producers (two warpgroups, half of each chunk) ----------------
+        // ---------------- producers (two warpgroups, alternate chunks) ----------------
         const int wg = warp >> 2;
         const int ptid = tid & 127;
         const uint32_t lane_base = uint32_t((warp & 3) * 32) << 16;
         bool ok = true;
         uint32_t jbase = 0;  // chunks of earlier units (stage ring position)
         uint32_t gbase = 0;  // accumulator groups of earlier units
-        uint32_t og = 0;     // symmetric mode: transposed products so far
-        uint32_t drained = 0;  // symmetric mode: transposed products drained so far
+        uint32_t og = 0;     // symmetric mode: transposed products of earlier units
         for (int64_t u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
             const TcInstance& I = batch.inst[SYM ? 0 : inst_of(batch, u)];
             const Unit un = SYM ? sym_unit_of(I, u) : unit_of(u - I.unit0, I.splits, I.nchunks, I.cps);
@@ -715,38 +713,42 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 tc_fence_before();
                 mbar_arrive(&dfree_bar[gg & 1]);
             };
-            // Symmetric mode: both warpgroups read the finished transposed
-            // accumulator of product m (buffer m & 1; M = 64 rows: row 16 q + l
-            // in lane l < 16 of the lane quarter q; warpgroup w the columns
-            // [8 w, 8 w + 8)) and store it as the FP32 partial sum of the 64
-            // sources of its chunk ch.
+            // Symmetric mode: the warpgroup that formed product m reads its
+            // finished transposed accumulator (buffer m & 1; M = 64 rows: row
+            // 16 q + l in lane l < 16 of the lane quarter q) and stores it as
+            // the FP32 partial sum of the 64 sources of its chunk ch.
             auto drain = [&](int64_t ch, uint32_t m) {
                 const int64_t p2 = sym_p2_index(int(ch), int(un.tile), I.sym_tile0, I.sym_tile1);
                 const bool got = ok && warp_wait(&d2full_bar[m & 1], (m >> 1) & 1u, wlim);
                 if (!got) ok = false;
                 tc_fence_after();
-                const int cb = wg * (NP / 2);
-                uint32_t v[8];
-                __syncwarp();
-                tmem_ld8(tmem + lane_base + uint32_t(kSymDJ + NP * int(m & 1) + cb), v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 // rows of kstride (k rounded up to 8) floats: two 16-byte
-                // stores per row and warpgroup
+                // stores per row and eight columns
                 const int kstride = (I.k_total + 7) & ~7;
-                if (got && lane < 16 && cb < kstride) {
-                    const int row = (warp & 3) * 16 + lane;
-                    float* dst = I.part2 + (p2 * 64 + row) * kstride + cb;
-                    st_global_v4(dst, v[0], v[1], v[2], v[3]);
-                    st_global_v4(dst + 4, v[4], v[5], v[6], v[7]);
+                const int row = (warp & 3) * 16 + lane;
+                float* dst = I.part2 + (p2 * 64 + row) * kstride;
+#pragma unroll 1
+                for (int cb = 0; cb < kstride; cb += 8) {
+                    uint32_t v[8];
+                    __syncwarp();
+                    tmem_ld8(tmem + lane_base + uint32_t(kSymDJ + NP * int(m & 1) + cb), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (got && lane < 16) {
+                        st_global_v4(dst + cb, v[0], v[1], v[2], v[3]);
+                        st_global_v4(dst + cb + 4, v[4], v[5], v[6], v[7]);
+                    }
                 }
                 tc_fence_before();
                 mbar_arrive(&d2free_bar[m & 1]);
             };
             const int first_offd = SYM ? int(2 * un.tile + 2 - un.c0) : un.nloc;  // local index
-            // One chunk: wait for its record and a free kernel-tile stage,
-            // evaluate, split, store into tensor memory (and, for a transposed
-            // product, into the shared-memory tile), arrive. OFFD is fixed per
-            // loop so that neither path tests it per source.
+            const int ndiag = first_offd < 0 ? 0 : (first_offd > un.nloc ? un.nloc : first_offd);
+            // One chunk: wait for its record, evaluate, split, store into
+            // tensor memory (and, for a transposed product, into the
+            // shared-memory tile), arrive. The stage is waited for when the
+            // first 16 (BF16) or 8 (TF32) sources of the chunk are evaluated:
+            // the tensor core reads the stage's last tile meanwhile. OFFD is
+            // fixed per loop so that neither path tests it per source.
             auto chunk_step = [&](int jl, auto offd_tag) -> bool {
                 constexpr bool OFFD = decltype(offd_tag)::value;
                 // group g is folded kFlushLag chunks after it ends, when the
@@ -759,23 +761,21 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 if (!ok) return false;
                 const uint32_t jg = jbase + uint32_t(jl);
                 const int ss = int(jg % SSTAGES), s = int(jg % kStages);
+                const uint32_t m = og + uint32_t(jl - ndiag);  // transposed product of this chunk
                 if (!warp_wait(&loaded_bar[ss], uint32_t((jg / SSTAGES) & 1), wlim)) return false;
-                if (jg >= kStages && !warp_wait(&tfree_bar[s], uint32_t(((jg / kStages) - 1) & 1), wlim)) return false;
-                if (OFFD && og >= 2 && !warp_wait(&gfree_bar[og & 1], ((og >> 1) - 1) & 1u, wlim)) return false;
-                const float* cx = reinterpret_cast<const float*>(smem + REC_BASE + ss * STAGE_BYTES + 2 * IMG) + wg * SW;
+                const float* cx = reinterpret_cast<const float*>(smem + REC_BASE + ss * STAGE_BYTES + 2 * IMG);
                 const uint32_t acol = uint32_t(kAColBase + s * kAColsPerStage);
                 // this thread's 16-byte rows of the shared-memory kernel tile
-                // (target ptid; sources wg SW + 16 half + 0..15)
-                uint8_t* grow = smem + (og & 1) * kSymGBytes + (wg * SW / 8) * kSymSrcGroupStride +
-                                (ptid / 8) * kSymTgtGroupStride + (ptid % 8) * 16;
+                // (target ptid; 16 sources per quarter of the chunk)
+                uint8_t* grow = smem + (m & 1) * kSymGBytes + (ptid / 8) * kSymTgtGroupStride + (ptid % 8) * 16;
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
+                for (int part = 0; part < 4; ++part) {
                     // 16 (BF16) or 8 (TF32) sources: four per 16-byte load of
                     // each coordinate, differences and squares two at a time
                     uint32_t hi[8], lo[8];
 #pragma unroll
                     for (int q4 = 0; q4 < (TF32 ? 2 : 4); ++q4) {
-                        const int j0 = (SW / 2) * half + 4 * q4;
+                        const int j0 = (KC / 4) * part + 4 * q4;
                         const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(cx + j0);
                         const ulonglong2 yv = *reinterpret_cast<const ulonglong2*>(cx + KC + j0);
                         const ulonglong2 zv = *reinterpret_cast<const ulonglong2*>(cx + 2 * KC + j0);
@@ -790,15 +790,26 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                             split_bf16(g2, g3, hi[2 * q4 + 1], lo[2 * q4 + 1]);
                         }
                     }
+                    if (part == 0) {
+                        if (jg >= kStages && !warp_wait(&tfree_bar[s], uint32_t(((jg / kStages) - 1) & 1), wlim))
+                            return false;
+                        if (OFFD && m >= 2 && !warp_wait(&gfree_bar[m & 1], ((m >> 1) - 1) & 1u, wlim)) return false;
+                    }
                     __syncwarp();
-                    tmem_st8(tmem + lane_base + acol + uint32_t(16 * wg + 8 * half), hi);
-                    tmem_st8(tmem + lane_base + acol + 32u + uint32_t(16 * wg + 8 * half), lo);
+                    tmem_st8(tmem + lane_base + acol + uint32_t(8 * part), hi);
+                    tmem_st8(tmem + lane_base + acol + 32u + uint32_t(8 * part), lo);
                     if (OFFD) {
-                        uint8_t* gr = grow + half * 2 * kSymSrcGroupStride;
+                        uint8_t* gr = grow + part * 2 * kSymSrcGroupStride;
                         st_shared_v4(gr, hi[0], hi[1], hi[2], hi[3]);
                         st_shared_v4(gr + kSymSrcGroupStride, hi[4], hi[5], hi[6], hi[7]);
                         st_shared_v4(gr + kSymGBytes / 2, lo[0], lo[1], lo[2], lo[3]);
                         st_shared_v4(gr + kSymGBytes / 2 + kSymSrcGroupStride, lo[4], lo[5], lo[6], lo[7]);
+                    }
+                    // the chunk two back, whose product has been read out of
+                    // the tile just waited for
+                    if (OFFD && part == 0 && jl >= ndiag + 2) {
+                        drain(un.c0 + (jl - 2), m - 2);
+                        if (!ok) return false;
                     }
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -807,30 +818,19 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 if (OFFD) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc_fence_before();
                 mbar_arrive(&full_bar[s]);
-                if (OFFD) {
-                    // transposed products are drained two behind: product
-                    // og - 2 has long finished, and its buffer is the one the
-                    // next product needs
-                    if (og >= drained + 2) {
-                        drain(un.c0 + (jl - 2), drained);
-                        ++drained;
-                    }
-                    ++og;
-                }
                 return true;
             };
-            const int ndiag = first_offd < 0 ? 0 : (first_offd > un.nloc ? un.nloc : first_offd);
-            int jl = 0;
-            for (; jl < ndiag && ok; ++jl)
+            // this warpgroup's chunks: those of its parity, counted over all
+            // units (chunk j uses stage j mod 2)
+            int jl = int((jbase ^ uint32_t(wg)) & 1u);
+            for (; jl < ndiag && ok; jl += 2)
                 if (!chunk_step(jl, std::false_type{})) ok = false;
             if constexpr (SYM) {
-                for (; jl < un.nloc && ok; ++jl)
+                for (; jl < un.nloc && ok; jl += 2)
                     if (!chunk_step(jl, std::true_type{})) ok = false;
-                // the unit's last (up to two) transposed products
-                while (ok && drained < og) {
-                    drain(un.c0 + (un.nloc - int(og - drained)), drained);
-                    ++drained;
-                }
+                // the warpgroup's last transposed product of the unit
+                if (ok && jl - 2 >= ndiag) drain(un.c0 + (jl - 2), og + uint32_t(jl - 2 - ndiag));
+                og += uint32_t(un.nloc - ndiag);
             }
             while (ok && flushed < ngroups) {
                 flush(flushed, flushed == ngroups - 1);
