@@ -33,7 +33,7 @@
 //   * The partial sums of each source split are reduced by a second kernel in
 //     a fixed order, which also applies sigma^2 and the per-target scale.
 //   * Coordinates are pre-scaled so that the kernel argument needs no
-//     multiplication (see gamma_scaled), and the hi/lo splits cost three
+//     multiplication (see coord_scale), and the hi/lo splits cost three
 //     (BF16) or two (TF32) instructions per value.
 //
 // Every mbarrier wait is bounded by a clock limit (about a second, or the
@@ -291,30 +291,23 @@ __device__ __forceinline__ void split_tf32(float g0, float g1, uint32_t& hi0, ui
     lo1 = __float_as_uint(l1);
 }
 
-// Kernel value without sigma^2 from pre-scaled coordinate differences: the
-// conversion multiplies every coordinate by c (c^2 = a log2(e) for the
-// Gaussian, c = a log2(e) otherwise), so the base-2 exponent is a plain sum.
+// What gamma2 takes of the z differences, two values: their squares (rounded),
+// or the differences themselves for the separable exponential.
 template <int KIND>
-__device__ __forceinline__ float gamma_scaled(float dx, float dy, float dz) {
-    if (KIND == KL_KERNEL_GAUSS) return ex2_approx(-fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-    if (KIND == KL_KERNEL_EXP_SEP) return ex2_approx(-(fabsf(dx) + fabsf(dy) + fabsf(dz)));
-    if (KIND == KL_KERNEL_EXP) return ex2_approx(-sqrt_approx(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
-    if (KIND == KL_KERNEL_MATERN32) {
-        // a r = r' ln 2 with r' = a log2(e) r
-        const float r = sqrt_approx(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-        return fmaf(0.69314718055994531f, r, 1.0f) * ex2_approx(-r);
-    }
-    return 1.0f;
+__device__ __forceinline__ uint64_t zterm2(uint64_t dz) {
+    return KIND == KL_KERNEL_EXP_SEP ? dz : f2mul(dz, dz);
 }
 
-// Two kernel values from packed pre-scaled differences (dx0, dx1), ...
+// Two kernel values from packed pre-scaled differences (dx0, dx1), (dy0, dy1)
+// and the z terms. The z term comes first, so that values do not depend on
+// whether it was formed per source or once for sources of equal z.
 template <int KIND>
-__device__ __forceinline__ void gamma2(uint64_t dx, uint64_t dy, uint64_t dz, float& g0, float& g1) {
+__device__ __forceinline__ void gamma2(uint64_t dx, uint64_t dy, uint64_t zt, float& g0, float& g1) {
     if (KIND == KL_KERNEL_EXP_SEP) {
         float x0, x1, y0, y1, z0, z1;
         up2(dx, x0, x1);
         up2(dy, y0, y1);
-        up2(dz, z0, z1);
+        up2(zt, z0, z1);
         g0 = ex2_approx(-(fabsf(x0) + fabsf(y0) + fabsf(z0)));
         g1 = ex2_approx(-(fabsf(x1) + fabsf(y1) + fabsf(z1)));
         return;
@@ -324,7 +317,7 @@ __device__ __forceinline__ void gamma2(uint64_t dx, uint64_t dy, uint64_t dz, fl
         return;
     }
     float r0, r1;
-    up2(f2fma(dz, dz, f2fma(dy, dy, f2mul(dx, dx))), r0, r1);
+    up2(f2fma(dy, dy, f2fma(dx, dx, zt)), r0, r1);
     if (KIND == KL_KERNEL_GAUSS) {
         g0 = ex2_approx(-r0);
         g1 = ex2_approx(-r1);
@@ -346,21 +339,26 @@ __device__ __forceinline__ void gamma2(uint64_t dx, uint64_t dy, uint64_t dz, fl
 // problems); other values of KIND fix it at compile time.
 constexpr int kKindAny = -1;
 template <int KIND>
-__device__ __forceinline__ void gamma2_k(int kind, uint64_t dx, uint64_t dy, uint64_t dz, float& g0, float& g1) {
+__device__ __forceinline__ uint64_t zterm2_k(int kind, uint64_t dz) {
+    if (KIND != kKindAny) return zterm2<(KIND == kKindAny ? KL_KERNEL_CONST : KIND)>(dz);
+    return kind == KL_KERNEL_EXP_SEP ? zterm2<KL_KERNEL_EXP_SEP>(dz) : zterm2<KL_KERNEL_GAUSS>(dz);
+}
+template <int KIND>
+__device__ __forceinline__ void gamma2_k(int kind, uint64_t dx, uint64_t dy, uint64_t zt, float& g0, float& g1) {
     if (KIND != kKindAny) {
-        gamma2<(KIND == kKindAny ? KL_KERNEL_CONST : KIND)>(dx, dy, dz, g0, g1);
+        gamma2<(KIND == kKindAny ? KL_KERNEL_CONST : KIND)>(dx, dy, zt, g0, g1);
         return;
     }
     switch (kind) {
-        case KL_KERNEL_GAUSS: gamma2<KL_KERNEL_GAUSS>(dx, dy, dz, g0, g1); break;
-        case KL_KERNEL_EXP_SEP: gamma2<KL_KERNEL_EXP_SEP>(dx, dy, dz, g0, g1); break;
-        case KL_KERNEL_EXP: gamma2<KL_KERNEL_EXP>(dx, dy, dz, g0, g1); break;
-        case KL_KERNEL_MATERN32: gamma2<KL_KERNEL_MATERN32>(dx, dy, dz, g0, g1); break;
-        default: gamma2<KL_KERNEL_CONST>(dx, dy, dz, g0, g1); break;
+        case KL_KERNEL_GAUSS: gamma2<KL_KERNEL_GAUSS>(dx, dy, zt, g0, g1); break;
+        case KL_KERNEL_EXP_SEP: gamma2<KL_KERNEL_EXP_SEP>(dx, dy, zt, g0, g1); break;
+        case KL_KERNEL_EXP: gamma2<KL_KERNEL_EXP>(dx, dy, zt, g0, g1); break;
+        case KL_KERNEL_MATERN32: gamma2<KL_KERNEL_MATERN32>(dx, dy, zt, g0, g1); break;
+        default: gamma2<KL_KERNEL_CONST>(dx, dy, zt, g0, g1); break;
     }
 }
 
-// Coordinate scale c of gamma_scaled: the argument a r^2 log2(e) (Gaussian) or
+// Coordinate scale c (every coordinate is multiplied by it): the argument a r^2 log2(e) (Gaussian) or
 // a r log2(e) (exponentials, Matern) becomes |c x - c y|^2 or |c x - c y|.
 float coord_scale(const KernelSpec& ks) {
     const double l2e = 1.4426950408889634074;
@@ -396,9 +394,16 @@ __host__ __device__ inline uint32_t img_offset(int n, int kk, int np, int esize)
 // of N <= 128 costs the same issue time whatever N is).
 __host__ __device__ constexpr bool tc_concat(bool tf32, int np) { return !tf32 && np == 16; }
 
+// Bytes of a chunk record: hi and lo image, x, y, z, and a float that is 1 when
+// all sources of the chunk have the same z (records are multiples of 128 bytes,
+// as the images' core matrices are).
+__host__ __device__ constexpr int tc_record_bytes(int np, int kchunk, int esize) {
+    return 2 * np * kchunk * esize + 12 * kchunk + 128;
+}
+
 // X (FP64) -> split images + FP32 source coordinates, chunk by chunk. A chunk
 // is one contiguous record [hi image | lo image | x[kchunk] y[kchunk]
-// z[kchunk]] (the stage layout), so that one bulk copy loads it; with the
+// z[kchunk] | flag] (the stage layout), so that one bulk copy loads it; with the
 // combined layout the two images form one image of 2 np rows.
 __global__ void tc_convert_kernel(const double* __restrict__ X, int64_t ldx, int64_t S, int c0, int kc,
                                   int np, int kchunk, bool tf32, float cscale, const float* __restrict__ sx,
@@ -407,7 +412,7 @@ __global__ void tc_convert_kernel(const double* __restrict__ X, int64_t ldx, int
     chain_wait();
     const int esize = tf32 ? 4 : 2;
     const int64_t img_bytes = int64_t(np) * kchunk * esize;  // one of hi / lo
-    const int64_t rec_bytes = 2 * img_bytes + 12 * int64_t(kchunk);
+    const int64_t rec_bytes = tc_record_bytes(np, kchunk, esize);
     const int64_t total = nchunks * kchunk * np;
     for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < total;
          t += int64_t(gridDim.x) * blockDim.x) {
@@ -418,6 +423,17 @@ __global__ void tc_convert_kernel(const double* __restrict__ X, int64_t ldx, int
         const float v = (s < S && n < kc) ? float(X[s + int64_t(c0 + n) * ldx]) : 0.f;
         uint8_t* base = img + ch * rec_bytes;
         const uint32_t off = img_offset(n, kk, np, esize);
+        if (t % (kchunk * np) < 32) {
+            // the chunk's first warp: points are ordered with the third
+            // direction slowest, so chunks of equal z are the rule (the
+            // padding behind the last source meets X = 0)
+            const int64_t first = ch * kchunk;
+            const float z0 = sz[first];
+            bool same = true;
+            for (int64_t q = first + (threadIdx.x & 31); q < first + kchunk && q < S; q += 32) same = same && sz[q] == z0;
+            same = __all_sync(0xffffffffu, same);
+            if (n == 0 && kk == 0) *reinterpret_cast<float*>(base + rec_bytes - 128) = same ? 1.0f : 0.0f;
+        }
         if (tc_concat(tf32, np)) {
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
             const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
@@ -551,7 +567,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
     constexpr int ESIZE = TF32 ? 4 : 2;
     constexpr int KC = TF32 ? 32 : 64;                  // sources per chunk (32 TMEM columns)
     constexpr int IMG = NP * KC * ESIZE;                // bytes of one of hi / lo
-    constexpr int STAGE_BYTES = 2 * IMG + KC * 12;      // hi, lo, coordinates x[KC] y[KC] z[KC]
+    constexpr int STAGE_BYTES = tc_record_bytes(NP, KC, ESIZE);  // hi, lo, x[KC] y[KC] z[KC], flag
     constexpr int SSTAGES = SYM ? kSymRecStages : smem_stages(STAGE_BYTES);  // shared-memory ring (>= kStages)
     constexpr int REC_BASE = SYM ? kSymRecBase : 0;
     constexpr uint32_t IDESC = instr_desc(NP, TF32);
@@ -768,6 +784,10 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 // this thread's 16-byte rows of the shared-memory kernel tile
                 // (target ptid; 16 sources per quarter of the chunk)
                 uint8_t* grow = smem + (m & 1) * kSymGBytes + (ptid / 8) * kSymTgtGroupStride + (ptid % 8) * 16;
+                auto parts = [&](auto samez_tag) -> bool {
+                constexpr bool SAMEZ = decltype(samez_tag)::value;
+                uint64_t zt = 0;
+                if (SAMEZ) zt = zterm2_k<KIND>(kind, f2sub(ppz, pk2(cx[2 * KC], cx[2 * KC])));
 #pragma unroll
                 for (int part = 0; part < 4; ++part) {
                     // 16 (BF16) or 8 (TF32) sources: four per 16-byte load of
@@ -778,10 +798,15 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                         const int j0 = (KC / 4) * part + 4 * q4;
                         const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(cx + j0);
                         const ulonglong2 yv = *reinterpret_cast<const ulonglong2*>(cx + KC + j0);
-                        const ulonglong2 zv = *reinterpret_cast<const ulonglong2*>(cx + 2 * KC + j0);
+                        uint64_t za = zt, zb = zt;
+                        if (!SAMEZ) {
+                            const ulonglong2 zv = *reinterpret_cast<const ulonglong2*>(cx + 2 * KC + j0);
+                            za = zterm2_k<KIND>(kind, f2sub(ppz, zv.x));
+                            zb = zterm2_k<KIND>(kind, f2sub(ppz, zv.y));
+                        }
                         float g0, g1, g2, g3;
-                        gamma2_k<KIND>(kind, f2sub(ppx, xv.x), f2sub(ppy, yv.x), f2sub(ppz, zv.x), g0, g1);
-                        gamma2_k<KIND>(kind, f2sub(ppx, xv.y), f2sub(ppy, yv.y), f2sub(ppz, zv.y), g2, g3);
+                        gamma2_k<KIND>(kind, f2sub(ppx, xv.x), f2sub(ppy, yv.x), za, g0, g1);
+                        gamma2_k<KIND>(kind, f2sub(ppx, xv.y), f2sub(ppy, yv.y), zb, g2, g3);
                         if (TF32) {
                             split_tf32(g0, g1, hi[4 * q4], hi[4 * q4 + 1], lo[4 * q4], lo[4 * q4 + 1]);
                             split_tf32(g2, g3, hi[4 * q4 + 2], hi[4 * q4 + 3], lo[4 * q4 + 2], lo[4 * q4 + 3]);
@@ -811,6 +836,16 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                         drain(un.c0 + (jl - 2), m - 2);
                         if (!ok) return false;
                     }
+                }
+                return true;
+                };
+                // sources of one z (nearly every chunk of a tensor grid): its
+                // term is formed once. Not in the symmetric form, which runs
+                // out of registers with both versions (16^3 cube, 627 -> 684 us)
+                if constexpr (SYM) {
+                    if (!parts(std::false_type{})) return false;
+                } else {
+                    if (!(cx[3 * KC] != 0.0f ? parts(std::true_type{}) : parts(std::false_type{}))) return false;
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 // generic-proxy stores to shared memory become visible to the
@@ -1002,7 +1037,7 @@ template <int KIND, bool TF32, int NP, bool SYM>
 cudaError_t launch_batch_np(const TcBatch& b, int sm_count, int* err, cudaStream_t s) {
     constexpr int ESIZE = TF32 ? 4 : 2;
     constexpr int KC = TF32 ? 32 : 64;
-    constexpr int STAGE_BYTES = 2 * NP * KC * ESIZE + KC * 12;
+    constexpr int STAGE_BYTES = tc_record_bytes(NP, KC, ESIZE);
     constexpr int ring = SYM ? kSymRecBase + kSymRecStages * STAGE_BYTES : smem_stages(STAGE_BYTES) * STAGE_BYTES;
     // at least ~100 KB so that no more than two CTAs share an SM (256 TMEM
     // columns each)
@@ -1247,7 +1282,7 @@ TcPlan plan(int64_t T, int64_t S, int k, int sm_count, bool tf32) {
     const int esize = tf32 ? 4 : 2;
     p.nblk = (k + 63) / 64;
     // one record per chunk: hi and lo images and the coordinates (16-byte multiple)
-    p.img_blk_doubles = (p.nchunks * (2 * p.np_max * p.kchunk * esize + 12 * p.kchunk) + 7) / 8;
+    p.img_blk_doubles = (p.nchunks * tc_record_bytes(p.np_max, p.kchunk, esize) + 7) / 8;
     p.img_doubles = p.nblk * p.img_blk_doubles;
     p.src_doubles = 0;  // coordinates are part of the chunk records
     p.part_doubles = int64_t(p.splits) * k * T;
@@ -1328,7 +1363,7 @@ cudaError_t tc_launch_batch(TcBatch& b, bool tf32, int np, int sm_count, int* er
 #ifdef KL_CHECK_BOUNDS
     {
         const int esize = tf32 ? 4 : 2, kchunk = tf32 ? 32 : 64;
-        const int64_t stage_bytes = 2 * int64_t(np) * kchunk * esize + 12 * int64_t(kchunk);
+        const int64_t stage_bytes = tc_record_bytes(np, kchunk, esize);
         for (int i = 0; i < b.ninst; ++i) {
             const TcInstance& I = b.inst[i];
             KL_RANGE(I.tx, I.T, float, "tc targets x");
@@ -1419,7 +1454,7 @@ TcSymPlan tc_sym_plan(int64_t T, int kcap, int sm_count) {
     // scratch: chunk records | unit table | direct partials (float2 per unit,
     // column and row) | transposed partials (float) | running sums (float2,
     // with more than one band)
-    const int stage_bytes = 2 * 16 * 64 * 2 + 64 * 12;
+    const int stage_bytes = tc_record_bytes(16, 64, 2);
     p.off_img = 0;
     p.off_tab = (p.nchunks * stage_bytes + 15) / 16 * 2;
     p.off_part1 = p.off_tab + (int64_t(p.nt) + 2) / 2 * 2;
