@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(256) gemm_tn_reduce(const double* __restrict__
 
 // ------------------------------- gemm_nn ----------------------------------
 constexpr int NN_C = 8;     // columns of C per block
+static_assert(NN_C >= kGemmNnInPlace, "in-place products need one block per row");
 constexpr int NN_R = 32;    // rows of C per block
 constexpr int NN_G = 8;     // threads sharing one row (the inner dimension split)
 constexpr int NN_MB = 128;  // rows of B staged per pass
@@ -164,7 +165,8 @@ constexpr int NN_MB = 128;  // rows of B staged per pass
 // C(K x n) = alpha A(K x m) B(m x n) + beta C: 32-row blocks so that the FP64
 // work (bound by each SM's FP64 rate) reaches every SM for K of a few thousand;
 // the 8 threads of a row take every 8th inner index and add up in shared memory.
-__global__ void __launch_bounds__(256) gemm_nn_kernel(const double* __restrict__ A, int64_t lda,
+// With n <= NN_C a block owns its rows, so that C may be A (beta = 0, m <= NN_MB).
+__global__ void __launch_bounds__(256) gemm_nn_kernel(const double* A, int64_t lda,
                                                       const double* __restrict__ B, int64_t ldb,
                                                       double* C, int64_t ldc, int64_t K, int m,
                                                       int n, double alpha, double beta) {
@@ -360,6 +362,66 @@ __global__ void __launch_bounds__(256) chol_rinv_smem_kernel(double* G, int n, d
     }
 }
 
+// One-warp form for n <= N (the blocks of the eigensolver: 8, 16): lane i holds
+// row i of L, then lane c column c of L^-1; broadcasts replace the block
+// barriers, several per column, that the chain of pivots otherwise waits for.
+// The same tests and operations as above. n = 8: 20.6 -> 11.1 us (cold).
+template <int N>
+__global__ void __launch_bounds__(32) chol_rinv_warp_kernel(double* G, int n, double* Rinv, int* bad) {
+    chain_wait();
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x;
+    double a[N], inv[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) a[j] = lane < n && j <= lane ? G[lane + int64_t(j) * n] : (j == lane ? 1.0 : 0.0);
+    const double g0 = lane < n ? G[lane + int64_t(lane) * n] : 0.0;
+    double maxd = fmax(g0, 0.0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) maxd = fmax(maxd, __shfl_xor_sync(kAll, maxd, o));
+    bool mine = false;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        inv[j] = 1.0;
+        if (j < n) {
+            const double d2 = __shfl_sync(kAll, a[j], j), gj = __shfl_sync(kAll, g0, j);
+            const bool b = !(d2 > 1e-28 * maxd) || !(d2 > 1e-14 * gj) || !isfinite(d2);
+            const double y = b ? 1.0 : rsqrt_newton(d2);
+            inv[j] = y;
+            if (lane == j) {
+                a[j] = b ? 1.0 : d2 * y;
+                mine = b;
+            } else if (lane > j) {
+                a[j] = b ? 0.0 : a[j] * y;
+            }
+#pragma unroll
+            for (int l = j + 1; l < N; ++l) {
+                const double f = __shfl_sync(kAll, a[j], l);
+                if (lane >= l) a[l] -= a[j] * f;
+            }
+        }
+    }
+    if (lane < n) {
+        bad[lane] = mine;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (j <= lane) G[lane + int64_t(j) * n] = a[j];
+    }
+    double x[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = i == lane ? 1.0 : 0.0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+        x[l] *= inv[l];
+#pragma unroll
+        for (int i = l + 1; i < N; ++i) x[i] -= __shfl_sync(kAll, a[l], i) * x[l];
+    }
+    if (lane < n) {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (i < n) Rinv[lane + int64_t(i) * n] = i >= lane ? x[i] : 0.0;
+    }
+}
+
 }  // namespace
 
 // Enough for every product with m' <= m, n' <= n and this K: a smaller
@@ -413,6 +475,11 @@ cudaError_t launch_chol_rinv(double* G, int n, double* Rinv, int* bad, cudaStrea
     KL_RANGE(G, int64_t(n) * n, double, "chol G");
     KL_RANGE(Rinv, int64_t(n) * n, double, "chol Rinv");
     KL_RANGE(bad, n, int, "chol flags");
+    if (n >= 1 && n <= 16) {
+        if (n <= 8) launch_chain(chol_rinv_warp_kernel<8>, 1, 32, 0, s, G, n, Rinv, bad);
+        else launch_chain(chol_rinv_warp_kernel<16>, 1, 32, 0, s, G, n, Rinv, bad);
+        return cudaGetLastError();
+    }
     if (n >= 1 && n <= kCholSmemN) {
         static std::once_flag once;
         static cudaError_t attr_error = cudaSuccess;

@@ -595,13 +595,13 @@ int64_t pair_scratch_doubles(int64_t T, int k, int splits) { return T * int64_t(
 
 int pair_choose_splits(int64_t T, int64_t S, int sm_count, bool fine) {
     // 16 blocks per SM while a split keeps 512 sources. `fine`: 256, and few
-    // sources are cut down to 16 per split for one wave of five blocks per SM
+    // sources are cut down to 4 per split for one wave of five blocks per SM
     // (216 targets and sources, one column, FP64: 250 us in one split per tile
-    // of targets, 12 us in 13); the partial sums take more memory, which
-    // handles that use this product for a refinement only do without.
+    // of targets, 12 us in 13, 10 us in 54); the partial sums take more memory,
+    // which handles that use this product for a refinement only do without.
     const int64_t tb = (T + kTgt - 1) / kTgt;
     const int64_t many = std::min<int64_t>((16LL * sm_count + tb - 1) / tb, S / (fine ? 256 : 512));
-    const int64_t few = fine ? std::min<int64_t>(5LL * sm_count / tb, S / 16) : 1;
+    const int64_t few = fine ? std::min<int64_t>(5LL * sm_count / tb, S / 4) : 1;
     return int(std::min<int64_t>(64, std::max<int64_t>(1, std::max(many, few))));
 }
 

@@ -241,7 +241,9 @@ cudaError_t launch_gemm_tn(const double* A, int64_t lda, const double* B, int64_
                            double* scratch, int64_t scratch_doubles, cudaStream_t s);
 // Scratch (doubles) of launch_gemm_tn for every m' <= m, n' <= n at this K.
 int64_t gemm_tn_scratch_doubles(int m, int n, int64_t K);
-// C(K x n) = alpha * A(K x m) B(m x n) + beta * C.
+// C(K x n) = alpha * A(K x m) B(m x n) + beta * C. C may be A for m = n <=
+// kGemmNnInPlace and beta = 0.
+constexpr int kGemmNnInPlace = 8;
 cudaError_t launch_gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, double* C,
                            int64_t ldc, int64_t K, int m, int n, double alpha, double beta,
                            cudaStream_t s);

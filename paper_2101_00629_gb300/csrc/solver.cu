@@ -139,6 +139,10 @@ int orthonormalize(Ctx& c, const double* V, int nv, double* W, int bw) {
         for (int pass = 0; pass < 2; ++pass) {
             KL_TRY(tn(c, W, c.N, W, c.N, c.w.G, bw, bw, bw));
             KL_TRY(ck(c, launch_chol_rinv(c.w.G, bw, c.w.Rinv, c.w.ibuf + pass * bw, c.h->stream), "chol"));
+            if (bw <= kGemmNnInPlace) {
+                KL_TRY(nn(c, W, c.N, c.w.Rinv, bw, W, c.N, bw, bw, 1.0, 0.0));
+                continue;
+            }
             KL_TRY(nn(c, W, c.N, c.w.Rinv, bw, c.w.T2, c.N, bw, bw, 1.0, 0.0));
             KL_TRY(ck(c, launch_copy_block(c.w.T2, c.N, W, c.N, c.N, bw, c.h->stream), "copy"));
         }
