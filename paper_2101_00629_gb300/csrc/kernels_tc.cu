@@ -230,6 +230,30 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
         : "memory");
 }
 
+template <int N>
+__device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t* v) {
+    static_assert(N == 4 || N == 8, "columns of a tensor-memory access");
+    if constexpr (N == 8) {
+        tmem_ld8(taddr, v);
+    } else {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                     : "r"(taddr)
+                     : "memory");
+    }
+}
+template <int N>
+__device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t* v) {
+    static_assert(N == 4 || N == 8, "columns of a tensor-memory access");
+    if constexpr (N == 8) {
+        tmem_st8(taddr, v);
+    } else {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]),
+                     "r"(v[1]), "r"(v[2]), "r"(v[3])
+                     : "memory");
+    }
+}
+
 __device__ __forceinline__ uint32_t tf32_rna(float x) {
     uint32_t y;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(x));
@@ -391,8 +415,13 @@ __host__ __device__ inline uint32_t img_offset(int n, int kk, int np, int esize)
 // A_hi [X_hi | X_lo] and a second of N = 16 (the first 16 rows) adds A_lo X_hi
 // into the first half: four MMAs per chunk instead of six. The issuing
 // thread, not the tensor core, limits the pipeline at these shapes (an MMA
-// of N <= 128 costs the same issue time whatever N is).
-__host__ __device__ constexpr bool tc_concat(bool tf32, int np) { return !tf32 && np == 16; }
+// of N <= 128 costs the same issue time whatever N is). With at most eight
+// vectors (np = 8) the image has 16 rows, [hi | lo] of eight each: A_hi and A_lo
+// both multiply the whole of it, N = 16, which adds the product of the two low
+// parts; the transposed products take two MMAs per K step instead of three, and
+// the folds half of the columns. 16^3 cube, symmetric form, whole application:
+// 627 -> 555 us.
+__host__ __device__ constexpr bool tc_concat(bool tf32, int np) { return !tf32 && np <= 16; }
 
 // Bytes of a chunk record: hi and lo image, x, y, z, and a float that is 1 when
 // all sources of the chunk have the same z (records are multiples of 128 bytes,
@@ -561,7 +590,8 @@ template <int KIND, bool TF32, int NP, bool SYM>
 __global__ void __launch_bounds__(kThreads, 2)
 pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
     chain_wait();
-    static_assert(!SYM || (!TF32 && NP == 16), "symmetric mode: split BF16, N = 16");
+    static_assert(!SYM || tc_concat(TF32, NP), "symmetric mode: split BF16, at most 16 vectors");
+    static_assert(NP >= 16 || tc_concat(TF32, NP), "an MMA of M = 128 has N >= 16");
     const int64_t nunits = batch.nunits;
     const long long wlim = batch.wait_limit > 0 ? batch.wait_limit : kWaitLimit;
     constexpr int ESIZE = TF32 ? 4 : 2;
@@ -570,17 +600,19 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
     constexpr int STAGE_BYTES = tc_record_bytes(NP, KC, ESIZE);  // hi, lo, x[KC] y[KC] z[KC], flag
     constexpr int SSTAGES = SYM ? kSymRecStages : smem_stages(STAGE_BYTES);  // shared-memory ring (>= kStages)
     constexpr int REC_BASE = SYM ? kSymRecBase : 0;
-    constexpr uint32_t IDESC = instr_desc(NP, TF32);
     constexpr bool kConcat = tc_concat(TF32, NP);
+    constexpr bool kNarrow = NP == 8;                   // [hi | lo] of eight columns each, N = 16
+    constexpr uint32_t IDESC = instr_desc(kNarrow ? 16 : NP, TF32);
+    constexpr int FC = NP / 2 < 8 ? NP / 2 : 8;         // columns of a fold step
     constexpr uint32_t IDESC2 = instr_desc(2 * NP, TF32);  // combined [hi | lo] operand
     // transposed product: M = 64 sources, A (kernel tile) MN-major
-    constexpr uint32_t IDESC_T = instr_desc_t64(NP);
+    constexpr uint32_t IDESC_T = instr_desc_t64(16);
     static_assert(!kConcat || 2 * NP <= TmemLayout<NP>::kDStride, "combined accumulator wider than its buffer");
     constexpr bool kSum = TmemLayout<NP>::kSum;
     constexpr int kDStride = TmemLayout<NP>::kDStride;
     constexpr int kSBase = TmemLayout<NP>::kSBase;
     constexpr int kAColBase = TmemLayout<NP>::kAColBase;
-    static_assert(!SYM || (kAColBase + kStages * kAColsPerStage <= kSymDJ && kSymDJ + 2 * NP <= kTmemCols),
+    static_assert(!SYM || (kAColBase + kStages * kAColsPerStage <= kSymDJ && kSymDJ + 2 * 16 <= kTmemCols),
                   "symmetric mode: tensor memory overflow");
 
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -675,25 +707,25 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 tc_fence_after();
                 const uint32_t dcol = uint32_t((gg & 1) * kDStride);
 #pragma unroll 1
-                for (int cb = wg * (NP / 2); cb < (wg + 1) * (NP / 2); cb += 8) {
-                    uint32_t v[8], h[8], l[8];
+                for (int cb = wg * (NP / 2); cb < (wg + 1) * (NP / 2); cb += FC) {
+                    uint32_t v[FC], h[FC], l[FC];
                     __syncwarp();
-                    tmem_ld8(tmem + lane_base + dcol + uint32_t(cb), v);
+                    tmem_ldn<FC>(tmem + lane_base + dcol + uint32_t(cb), v);
                     if (kConcat) {
-                        uint32_t v2[8];
-                        tmem_ld8(tmem + lane_base + dcol + uint32_t(NP + cb), v2);
+                        uint32_t v2[FC];
+                        tmem_ldn<FC>(tmem + lane_base + dcol + uint32_t(NP + cb), v2);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)
+                        for (int q = 0; q < FC; ++q)
                             v[q] = __float_as_uint(__fadd_rn(__uint_as_float(v[q]), __uint_as_float(v2[q])));
                     }
                     if (kSum && g > 0) {
-                        tmem_ld8(tmem + lane_base + uint32_t(kSBase + cb), h);
-                        tmem_ld8(tmem + lane_base + uint32_t(kSBase + NP + cb), l);
+                        tmem_ldn<FC>(tmem + lane_base + uint32_t(kSBase + cb), h);
+                        tmem_ldn<FC>(tmem + lane_base + uint32_t(kSBase + NP + cb), l);
                     }
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
+                    for (int q = 0; q < FC; ++q) {
                         const float x = __uint_as_float(v[q]);
                         float hs = x, ls = 0.f;
                         if (kSum) {
@@ -715,11 +747,11 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                         l[q] = __float_as_uint(ls);
                     }
                     if (kSum && !last) {
-                        tmem_st8(tmem + lane_base + uint32_t(kSBase + cb), h);
-                        tmem_st8(tmem + lane_base + uint32_t(kSBase + NP + cb), l);
+                        tmem_stn<FC>(tmem + lane_base + uint32_t(kSBase + cb), h);
+                        tmem_stn<FC>(tmem + lane_base + uint32_t(kSBase + NP + cb), l);
                     } else if (got && t < T) {
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)
+                        for (int q = 0; q < FC; ++q)
                             if (cb + q < kc)
                                 prow[int64_t(cb + q) * pstride] =
                                     make_float2(__uint_as_float(h[q]), __uint_as_float(l[q]));
@@ -744,10 +776,18 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                 const int row = (warp & 3) * 16 + lane;
                 float* dst = I.part2 + (p2 * 64 + row) * kstride;
 #pragma unroll 1
-                for (int cb = 0; cb < kstride; cb += 8) {
+                for (int cb = 0; cb < (kNarrow ? 8 : kstride); cb += 8) {
                     uint32_t v[8];
                     __syncwarp();
-                    tmem_ld8(tmem + lane_base + uint32_t(kSymDJ + NP * int(m & 1) + cb), v);
+                    tmem_ld8(tmem + lane_base + uint32_t(kSymDJ + 16 * int(m & 1) + cb), v);
+                    if (kNarrow) {
+                        uint32_t v2[8];
+                        tmem_ld8(tmem + lane_base + uint32_t(kSymDJ + 16 * int(m & 1) + 8), v2);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            v[q] = __float_as_uint(__fadd_rn(__uint_as_float(v[q]), __uint_as_float(v2[q])));
+                    }
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (got && lane < 16) {
                         st_global_v4(dst + cb, v[0], v[1], v[2], v[3]);
@@ -917,9 +957,9 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                         const uint32_t ah = acol + uint32_t(ks * 8), al = acol + 32u + uint32_t(ks * 8);
                         if (kConcat) {
                             // rows 0..2NP-1 of the combined image: [X_hi | X_lo];
-                            // its first NP rows: X_hi
+                            // its first NP rows: X_hi (kNarrow: all 16 rows)
                             const uint64_t bb = bst + uint64_t((ks * kStep) >> 4);
-                            mma_tmemA(TF32, d_tmem, ah, bb, IDESC2, (first && ks == 0) ? 0u : 1u);
+                            mma_tmemA(TF32, d_tmem, ah, bb, kNarrow ? IDESC : IDESC2, (first && ks == 0) ? 0u : 1u);
                             mma_tmemA(TF32, d_tmem, al, bb, IDESC, 1u);
                         } else {
                             const uint64_t bh = bst + uint64_t((ks * kStep) >> 4);
@@ -945,7 +985,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                         tc_fence_after();
                         const uint64_t gd = gdesc0 + uint64_t(uint32_t((m & 1) * kSymGBytes) >> 4);
                         const uint64_t xd = xdesc0 + uint64_t(uint32_t(xb * kSymXBytes) >> 4);
-                        const uint32_t dj = tmem + uint32_t(kSymDJ + NP * int(m & 1));
+                        const uint32_t dj = tmem + uint32_t(kSymDJ + 16 * int(m & 1));
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {
                             // K step ks: targets 16 ks .. 16 ks + 15 (two core
@@ -956,7 +996,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                             const uint64_t bh = xd + uint64_t((ks * kStep) >> 4);
                             const uint64_t bl = bh + uint64_t((NP / 8 * 128) >> 4);
                             mma_smemA(dj, ah, bh, IDESC_T, ks == 0 ? 0u : 1u);
-                            mma_smemA(dj, ah, bl, IDESC_T, 1u);
+                            if (!kNarrow) mma_smemA(dj, ah, bl, IDESC_T, 1u);
                             mma_smemA(dj, al, bh, IDESC_T, 1u);
                         }
                         mma_commit(&gfree_bar[m & 1]);
@@ -995,7 +1035,7 @@ pair_tc_kernel(const __grid_constant__ TcBatch batch, int* __restrict__ err) {
                     const uint32_t xb = xu & 1u;
                     if (xu >= 2 && !mbar_wait(&xfree_bar[xb], ((xu >> 1) - 1) & 1u, wlim)) { ok = false; break; }
                     uint8_t* dst = smem + 2 * kSymGBytes + xb * kSymXBytes;
-                    mbar_arrive_expect_tx(&xload_bar[xb], uint32_t(kSymXBytes));
+                    mbar_arrive_expect_tx(&xload_bar[xb], uint32_t(4 * IMG));
                     bulk_g2s(dst, img + 2 * un.tile * int64_t(STAGE_BYTES), uint32_t(2 * IMG), &xload_bar[xb]);
                     bulk_g2s(dst + 2 * IMG, img + (2 * un.tile + 1) * int64_t(STAGE_BYTES), uint32_t(2 * IMG),
                              &xload_bar[xb]);
@@ -1056,7 +1096,9 @@ cudaError_t launch_batch_np(const TcBatch& b, int sm_count, int* err, cudaStream
 template <int KIND, bool TF32>
 cudaError_t launch_batch_kind(const TcBatch& b, int np, bool sym, int sm_count, int* err, cudaStream_t s) {
     if constexpr (!TF32) {
-        if (sym) return launch_batch_np<KIND, false, 16, true>(b, sm_count, err, s);
+        if (sym) return np == 8 ? launch_batch_np<KIND, false, 8, true>(b, sm_count, err, s)
+                                : launch_batch_np<KIND, false, 16, true>(b, sm_count, err, s);
+        if (np == 8) return launch_batch_np<KIND, false, 8, false>(b, sm_count, err, s);
     }
     switch (np) {
         case 16: return launch_batch_np<KIND, TF32, 16, false>(b, sm_count, err, s);
@@ -1270,7 +1312,7 @@ TcPlan plan(int64_t T, int64_t S, int k, int sm_count, bool tf32) {
     p.kchunk = tf32 ? 32 : 64;
     p.nchunks = std::max<int64_t>(1, (S + p.kchunk - 1) / p.kchunk);
     const int kmax = std::min(k, 64);
-    p.np_max = std::max(16, (kmax + 15) / 16 * 16);
+    p.np_max = !tf32 && kmax <= 8 ? 8 : std::max(16, (kmax + 15) / 16 * 16);
     const int64_t tiles = (T + 127) / 128;
     const int64_t grid = 2LL * sm_count;
     int64_t want = (16 * grid + tiles - 1) / tiles;
@@ -1477,6 +1519,7 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
     if (a.tf32 || a.k < 1 || a.k > p.kcap || a.T != p.T || a.S != p.T || a.scratch_len < p.total)
         return cudaErrorInvalidValue;
     const float cscale = coord_scale(a.ks);
+    const int np = a.k <= 8 ? 8 : 16;
     uint8_t* img = reinterpret_cast<uint8_t*>(a.scratch + p.off_img);
     const int2* tab = reinterpret_cast<const int2*>(a.scratch + p.off_tab);
     float2* part1 = reinterpret_cast<float2*>(a.scratch + p.off_part1);
@@ -1490,9 +1533,9 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
     KL_RANGE(a.Y, block_extent(a.T, a.k, a.ldy), double, "tc sym Y");
     KL_RANGE(a.post, a.T, double, "tc sym post");
     {
-        const int64_t total = p.nchunks * 64 * 16;
+        const int64_t total = p.nchunks * 64 * np;
         const int g = int(std::min<int64_t>((total + 255) / 256, int64_t(a.sm_count) * 64));
-        launch_chain(tc_convert_kernel, g, 256, 0, s, a.X, a.ldx, a.S, 0, a.k, 16, 64, false, cscale, a.sx, a.sy, a.sz, img,
+        launch_chain(tc_convert_kernel, g, 256, 0, s, a.X, a.ldx, a.S, 0, a.k, np, 64, false, cscale, a.sx, a.sy, a.sz, img,
                                             p.nchunks);
         ++*launched;
         cudaError_t e = cudaGetLastError();
@@ -1544,7 +1587,7 @@ cudaError_t launch_pair_tc_sym(const TcArgs& a, cudaStream_t s, int* launched) {
             KL_RANGE(a.err, 1, int, "tc error word");
         }
 #endif
-        cudaError_t e = launch_batch_prec<false>(batch, 16, true, a.grid_sms > 0 ? a.grid_sms : a.sm_count, a.err, s);
+        cudaError_t e = launch_batch_prec<false>(batch, np, true, a.grid_sms > 0 ? a.grid_sms : a.sm_count, a.err, s);
         ++*launched;
         if (e != cudaSuccess) return e;
         // one block per chunk of the band's points and the later ones
