@@ -255,21 +255,28 @@ int ensure_workspace(kl_solver* h, int k) {
     cudaError_t e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "workspace sync");
     clear_graphs(h);
-    dfree(h->work);
+    for (double*& w : h->work) {
+        dfree(w);
+        w = nullptr;
+    }
     h->dev_bytes -= h->work_len * int64_t(sizeof(double));
-    h->work = nullptr;
     h->work_len = 0;
     h->k_cap = 0;
-    // one allocation for the three operator blocks and the pairwise scratch:
-    // each of them costs tens of microseconds of handle creation
+    // the three operator blocks and the pairwise scratch: one allocation where
+    // they are large (each costs tens of microseconds of handle creation), four
+    // where they fit the blocks that the driver cuts small allocations from
     const int64_t big = (std::max(h->S, h->T) * int64_t(k) + 31) / 32 * 32;
     h->pair_splits = pair_choose_splits(h->T, h->S, h->sm_count, cuda_cores(h->prm.precision));
     const int64_t scratch = std::max<int64_t>(pair_scratch_doubles(h->T, k, h->pair_splits),
                                               tc_scratch_doubles(h->T, h->S, k, h->sm_count));
-    if ((e = dalloc(h, &h->work, 3 * big + scratch)) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
-    h->work_len = 3 * big + scratch;
-    for (int i = 0; i < 3; ++i) h->ws[i] = h->work + i * big;
-    h->pair_scratch = h->work + 3 * big;
+    const bool small = std::max(big, scratch) * int64_t(sizeof(double)) <= int64_t(1) << 20;
+    const int64_t part[4] = {small ? big : 3 * big + scratch, big, big, scratch};
+    for (int i = 0; i < (small ? 4 : 1); ++i) {
+        if ((e = dalloc(h, &h->work[i], part[i])) != cudaSuccess) return cuda_fail(h, e, "workspace alloc");
+        h->work_len += part[i];
+    }
+    for (int i = 0; i < 3; ++i) h->ws[i] = small ? h->work[i] : h->work[0] + i * big;
+    h->pair_scratch = small ? h->work[3] : h->work[0] + 3 * big;
     h->pair_scratch_len = scratch;
     h->k_cap = k;
     return KL_OK;
@@ -1253,7 +1260,7 @@ int kl_destroy(kl_solver* h) {
     dfree(h->d_rat);
     dfree(h->d_band_vals);
     dfree(h->d_band_start);
-    dfree(h->work);
+    for (double* w : h->work) dfree(w);
     dfree(h->sym_scratch);
     delete h->sym_plan;
     dfree(h->eig_ws);

@@ -90,7 +90,7 @@ struct kl_solver {
 
     // workspaces for operator applications (k_cap vectors)
     int k_cap = 0;
-    double* work = nullptr;  // one allocation of work_len doubles: ws, pair_scratch
+    double* work[4] = {};  // allocations of ws and pair_scratch, work_len doubles in all
     int64_t work_len = 0;
     double* ws[3] = {nullptr, nullptr, nullptr};
     double* pair_scratch = nullptr;

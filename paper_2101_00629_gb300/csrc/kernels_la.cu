@@ -447,10 +447,10 @@ cudaError_t launch_gemm_tn(const double* A, int64_t lda, const double* B, int64_
     const int64_t kchunk = ((K + splits - 1) / splits + TN_T - 1) / TN_T * TN_T;
     if (n <= TN_NARROW) {
         dim3 grid((m + TN_T - 1) / TN_T, 1, splits);
-        launch_chain(gemm_tn_narrow_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
+        launch_kernel(short_fp64(double(K) * m * n), gemm_tn_narrow_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
     } else {
         dim3 grid((m + TN_T - 1) / TN_T, (n + TN_T - 1) / TN_T, splits);
-        launch_chain(gemm_tn_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
+        launch_kernel(short_fp64(double(K) * m * n), gemm_tn_kernel, grid, 256, 0, s, A, lda, B, ldb, m, n, K, kchunk, scratch);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -467,7 +467,7 @@ cudaError_t launch_gemm_nn(const double* A, int64_t lda, const double* B, int64_
     KL_RANGE(B, block_extent(m, n, ldb), double, "gemm_nn B");
     KL_RANGE(C, block_extent(K, n, ldc), double, "gemm_nn C");
     dim3 grid(unsigned((K + NN_R - 1) / NN_R), unsigned((n + NN_C - 1) / NN_C));
-    launch_chain(gemm_nn_kernel, grid, 256, 0, s, A, lda, B, ldb, C, ldc, K, m, n, alpha, beta);
+    launch_kernel(short_fp64(double(K) * m * n), gemm_nn_kernel, grid, 256, 0, s, A, lda, B, ldb, C, ldc, K, m, n, alpha, beta);
     return cudaGetLastError();
 }
 

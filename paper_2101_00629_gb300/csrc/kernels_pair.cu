@@ -601,7 +601,11 @@ int pair_choose_splits(int64_t T, int64_t S, int sm_count, bool fine) {
     // which handles that use this product for a refinement only do without.
     const int64_t tb = (T + kTgt - 1) / kTgt;
     const int64_t many = std::min<int64_t>((16LL * sm_count + tb - 1) / tb, S / (fine ? 256 : 512));
-    const int64_t few = fine ? std::min<int64_t>(5LL * sm_count / tb, S / 4) : 1;
+    int64_t few = fine ? std::min<int64_t>(5LL * sm_count / tb, S / 4) : 1;
+    // up to 1024 targets: partial sums of eight columns within 1 MiB, which is
+    // cheaper to allocate than more
+    const int64_t in_mib = (int64_t(1) << 17) / (8 * T);
+    if (in_mib >= 16) few = std::min(few, in_mib);
     return int(std::min<int64_t>(64, std::max<int64_t>(1, std::max(many, few))));
 }
 

@@ -524,10 +524,10 @@ cudaError_t launch_modeprod(const double* A, int m, int n, const double* X, int6
     KL_RANGE(pre, a * n * b, double, "modeprod pre");
     const int64_t per_col = a * m * b;
     if (per_col < (int64_t(1) << 31))
-        launch_chain(modeprod_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint32_t(a),
+        launch_kernel(short_fp64(double(per_col) * k * n), modeprod_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint32_t(a),
                                                                              uint32_t(b), k, post, pre);
     else
-        launch_chain(modeprod_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint64_t(a),
+        launch_kernel(short_fp64(double(per_col) * k * n), modeprod_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, A, m, n, X, ldx, Y, ldy, uint64_t(a),
                                                                              uint64_t(b), k, post, pre);
     return cudaGetLastError();
 }
@@ -545,10 +545,10 @@ cudaError_t launch_modeprod_band(const Band& A, int m, int n, const double* X, i
     KL_RANGE(pre, a * n * b, double, "band modeprod pre");
     const int64_t per_col = a * m * b;
     if (per_col < (int64_t(1) << 31))
-        launch_chain(modeprod_band_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, 
+        launch_kernel(short_fp64(double(per_col) * k * A.w), modeprod_band_kernel<uint32_t>, grid_cols(per_col, k), kThreads, 0, s, 
             A.vals, A.start, A.w, m, n, X, ldx, Y, ldy, uint32_t(a), uint32_t(b), k, post, pre);
     else
-        launch_chain(modeprod_band_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, 
+        launch_kernel(short_fp64(double(per_col) * k * A.w), modeprod_band_kernel<uint64_t>, grid_cols(per_col, k), kThreads, 0, s, 
             A.vals, A.start, A.w, m, n, X, ldx, Y, ldy, uint64_t(a), uint64_t(b), k, post, pre);
     return cudaGetLastError();
 }
