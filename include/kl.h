@@ -109,7 +109,9 @@ enum { KL_GALERKIN_IBQ = 0, KL_COLLOCATION = 1, KL_GALERKIN_STD = 2 };
  * symmetric Galerkin problems, the one that finds all wanted residuals below
  * the tolerance) are solved in FP32, and the returned pairs come from the
  * FP64 Rayleigh-Ritz refinement (`refine`).
- *   KL_FP64        FP64 kernel evaluation and products (CUDA cores).
+ *   KL_FP64        kernel values and products to FP64 accuracy (CUDA cores:
+ *                  64-bit fixed point where that is no less exact than FP64
+ *                  arithmetic, FP64 elsewhere).
  *   KL_FP32        FP32 kernel evaluation and FP32 products (CUDA cores).
  *   KL_MIXED_BF16  FP32 kernel tiles written to tensor memory and multiplied
  *                  on tcgen05 tensor cores as split (hi + lo) BF16 products
@@ -180,8 +182,9 @@ int kl_apply_A(kl_solver* h, const double* X, int64_t ldx, double* Y, int64_t ld
 
 /* Y = Z^-1 X (device FP64 blocks as above). Galerkin: Z^-1 = L^-T L^-1 with
  * the Kronecker Cholesky factor L = L_d x ... x L_1 (Sec. 3.1). Collocation:
- * the Kronecker pivoted-LU solve Z^-1 = Q U^-1 L^-1 P per direction
- * (Sec. 3.2, Sec. 3.3 Remark). X and Y may be the same buffer. */
+ * the Kronecker LU solve per direction (Sec. 3.2, Sec. 3.3 Remark: Z^-1 = Q U^-1
+ * L^-1 P; the totally positive 1D factors need no pivoting where they are
+ * applied as banded sweeps). X and Y may be the same buffer. */
 int kl_apply_Zinv(kl_solver* h, const double* X, int64_t ldx, double* Y, int64_t ldy, int k);
 
 /* Y = A' X with the standard-form operator of Eq. standard:
@@ -254,7 +257,7 @@ int kl_memory(const kl_solver* h, int64_t* h2d_bytes, int64_t* device_bytes);
  * Errors: KL_ERR_CUDA, KL_ERR_OOM. */
 int kl_measure_peaks(double* fp32_fma_per_s, double* ex2_per_s, double* fp64_fma_per_s);
 
-/* Y = sigma^2 Gamma(targets, sources) X with FP64 kernel evaluation on the
+/* Y = sigma^2 Gamma(targets, sources) X to FP64 accuracy (as KL_FP64) on the
  * CUDA cores, allocating no device memory. No paper passage: the paper has no
  * counterpart; this entry point exists for callers that cannot allocate --
  * code inside CUDA graph capture, applications with fixed memory pools, or

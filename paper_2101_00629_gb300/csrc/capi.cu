@@ -441,7 +441,8 @@ static int pairwise(kl_solver* h, int precision, const double* U, double* W, int
         a.scratch = h->pair_scratch; a.splits = h->pair_splits;
         ProfScope ps(h, precision == KL_FP64 ? "pair_f64" : "pair_f32", pairs);
         cudaError_t e = launch_pair_simt(a, precision == KL_FP32, h->stream);
-        h->launches += (k + 31) / 32 + 1;
+        const int step = precision == KL_FP64 && h->prm.kernel != KL_KERNEL_CONST ? 16 : 32;  // columns per pass
+        h->launches += (k + step - 1) / step + 1;
         if (e != cudaSuccess) return cuda_fail(h, e, "pairwise (CUDA cores)");
         return KL_OK;
     }
