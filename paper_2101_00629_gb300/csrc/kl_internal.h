@@ -121,7 +121,8 @@ int device_sm_count();
 // Launches that follow a wait for another stream's event are plain (chained
 // false), and so are the CUDA-core pairwise products with more blocks than
 // SMs: their blocks, placed while the predecessor still holds some SMs, would
-// crowd the others for the whole product (FP32 product 205 -> 286 us). The error, if any, is the one cudaGetLastError returns.
+// crowd the others for the whole product (FP32 product 205 -> 286 us). The
+// error, if any, is the one cudaGetLastError returns.
 // Measured: FP64 application of 216 dofs (8 kernels) 38.9 -> 23.7 us, FP64
 // solve of 8 pairs with 720 dofs (440 kernels) 9.34 -> 8.40 ms.
 __device__ __forceinline__ void chain_wait() {
