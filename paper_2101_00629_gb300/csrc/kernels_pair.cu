@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     __shared__ __align__(16) double s_xd[ST][KB];
     __shared__ float s_box[NG][6];
     __shared__ int s_emax[NG][KB];
-    __shared__ int s_special[NG], s_count[NG];
+    __shared__ int s_special[NG], s_count[NG], s_emin[NG];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < 1024; i += kTgt)
         reinterpret_cast<ulonglong2*>(s_tab)[i] = reinterpret_cast<const ulonglong2*>(g_exp2.v)[i];
@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             }
             float lo[3] = {float(x - rx) * sc.f, float(y - ry) * sc.f, float(z - rz) * sc.f}, hi[3];
             bool bad = !(isfinite(lo[0]) && isfinite(lo[1]) && isfinite(lo[2]));
+            int emin = 2047;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 hi[q] = lo[q];
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 int emax = __reduce_max_sync(0xffffffffu, e);
                 bad = bad || emax == 2047 || (emax > 0 && emax < 700);
                 if (emax == 0) emax = 1079;
+                emin = min(emin, emax);
                 // |x| 2^(1078 - emax), rounded: at most 2^56
                 const uint64_t m = ((b & 0xfffffffffffffull) | (ef ? uint64_t(1) << 52 : 0)) << 3;
                 const int rs = emax - e;
@@ -227,6 +229,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             if (lane == 0) {
                 s_special[g] = any_bad;
                 s_count[g] = __popc(have);
+                s_emin[g] = emin;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) s_box[g][q] = lo[q], s_box[g][3 + q] = hi[q];
             }
@@ -262,7 +265,9 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             tlo = fmaxf(tlo * (1.0f - 1e-5f) - 1e-3f, 0.0f);
             thi = thi * (1.0f + 1e-5f) + 1e-3f;
             const int n0 = int(fminf(tlo, 1000.0f));
-            const bool narrow = thi - float(n0) < most;
+            // the group's scale 2^(emax - 56 - n0) is a normal number in every
+            // column (far Gaussian groups: n0 reaches 999)
+            const bool narrow = thi - float(n0) < most && n0 <= s_emin[g] - 57;
             if (__all_sync(0xffffffffu, in_range && narrow)) {
                 int64_t hi[KB], mid[KB];
 #pragma unroll

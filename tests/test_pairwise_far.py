@@ -1,0 +1,91 @@
+"""FP64 pairwise products of points many correlation lengths apart: every value
+to its own size, wherever the kernel's exponent lies in the range of the
+fixed-point evaluation or beyond it (a sum over near and far pairs would hide
+the far ones). GPU against long double."""
+import numpy as np
+import pytest
+
+from oracle import galerkin
+from oracle.problem import Problem
+
+LN2 = np.log(2.0)
+
+
+def _exponent(kernel, L, d):
+    """-log of the kernel's exponential factor in long double; d: (3, ...)."""
+    L = np.longdouble(L)
+    d = np.abs(d.astype(np.longdouble))
+    if kernel == "exp_sep":
+        return d.sum(0) / L
+    if kernel == "gauss":
+        return (d ** 2).sum(0) / L ** 2
+    a = np.sqrt((d ** 2).sum(0)) / L
+    return np.sqrt(np.longdouble(3)) * a if kernel == "matern32" else a
+
+
+def _product(kernel, L, tgt, src, X):
+    import torch
+    import paper_2101_00629_gb300 as kl
+    d = [torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda() for a in (tgt, src, X)]
+    T, S, k = tgt.shape[1], src.shape[1], X.shape[0]
+    Y = torch.empty(k, T, dtype=torch.float64, device="cuda")
+    kl.kl_pairwise_noalloc(kernel, 1.0, L, d[0], T, d[1], S, d[2], S, Y, T, k, torch.cuda.current_stream())
+    return Y.cpu().numpy()
+
+
+def _check(kernel, L, tgt, src, X):
+    Y = _product(kernel, L, tgt, src, X)
+    a = _exponent(kernel, L, tgt[:, :, None] - src[:, None, :])
+    G = np.exp(-a) * (1 + a if kernel == "matern32" else 1)
+    Xl = X.astype(np.longdouble)
+    ref = Xl @ G.T
+    # what an FP64 evaluation may lose: rounding of the exponent a (a few
+    # 2^-53 a), of the value and of the sum; one unit of the subnormal range
+    # per term
+    bound = np.abs(Xl) @ ((16 + 4 * a) * G).T * 2.0 ** -53 + src.shape[1] * 2.0 ** -1073
+    assert np.all(np.isfinite(Y))
+    assert np.all(np.abs(Y - ref) <= bound)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("entry", [1.0, -1e-30, 1e-60, 1e-95])
+@pytest.mark.parametrize("base", [600, 700, 767, 768, 900, 966, 967, 968, 985, 999])
+def test_gaussian_group_scale(base, entry):
+    """Groups that are narrow far away: a single point, a compact group of 32,
+    and a group of one point behind a full one."""
+    r = np.sqrt((base + np.linspace(0.0, 0.9, 5)) * LN2)
+    tgt = np.zeros((3, 5))
+    tgt[0] = r
+    for S in (1, 32, 33):
+        src = np.zeros((3, S))
+        src[1] = 0.01 * np.arange(S) / 32
+        X = np.zeros((2, S))
+        X[0, -1] = entry
+        X[1] = entry * (1.0 + np.arange(S) / 64)
+        for t in range(5):  # one target at a time: a warp takes one path
+            _check("gauss", 1.0, tgt[:, t:t + 1], src, X)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("geometry,L", [("cube", 0.066), ("cube", 0.05), ("annulus", 0.115), ("annulus", 0.105)])
+def test_gaussian_operator_of_short_length(geometry, L):
+    """Corner groups of a grid with 4 m + 1 points hold one point and are narrow
+    at any distance."""
+    import torch
+    import paper_2101_00629_gb300 as kl
+    prob = Problem(geometry, 2, (7, 7, 7), "gauss", 1.0, L)
+    A, _, parts = galerkin.matrices(prob, with_parts=True)
+    Q = np.linalg.solve(parts["Bt"].T, parts["M"])
+    absA = np.abs(Q).T @ (parts["J"][:, None] * parts["Gamma"] * parts["J"][None, :]) @ np.abs(Q)
+    h = kl.kl_create(kl.params(geometry=geometry, degree=2, elems=(7, 7, 7), kernel="gauss", L=L, method="galerkin",
+                               precision="fp64"), torch.cuda.current_stream())
+    try:
+        N, _, _ = kl.kl_dims(h)
+        X = np.random.default_rng(5).standard_normal((3, N))
+        Xd = torch.from_numpy(X).cuda()
+        Y = torch.empty_like(Xd)
+        kl.kl_apply_A(h, Xd, N, Y, N, 3)
+        err = np.abs(Y.cpu().numpy() - (A @ X.T).T)
+        assert np.all(err <= 1e-12 * (absA @ np.abs(X).T).T)
+    finally:
+        kl.kl_destroy(h)
