@@ -25,14 +25,17 @@ namespace kl {
 namespace fx {
 
 // Fraction bits of the coordinates (kCoord) and of the exponent t (kArg).
-// Gauss: |difference| < 64, t = sum of squares < 2048. Others: t < 512; the
-// Euclidean ones need every |difference| < 128.
+// A coordinate difference is a signed 64-bit number: it is right for
+// |difference| < 64 (Gauss) or 256. kMaxArg keeps each difference and the
+// exponent in range, with room for the rounding of the bounds: Gauss t < 2048,
+// |difference| <= sqrt(1000); separable exponential t < 512, |difference| <= t;
+// Euclidean ones |difference| < 128 (the norm scales three squares to 62 bits).
 template <int KIND>
 struct Format {
     static constexpr int kCoord = KIND == KL_KERNEL_GAUSS ? 57 : 55;
     static constexpr int kArg = KIND == KL_KERNEL_GAUSS ? 53 : 55;
     // largest exponent the fixed-point evaluation takes
-    static constexpr float kMaxArg = KIND == KL_KERNEL_GAUSS ? 1000.0f : KIND == KL_KERNEL_EXP_SEP ? 500.0f : 120.0f;
+    static constexpr float kMaxArg = KIND == KL_KERNEL_GAUSS ? 1000.0f : KIND == KL_KERNEL_EXP_SEP ? 250.0f : 120.0f;
 };
 
 __host__ __device__ inline uint32_t mulhi32(uint32_t a, uint32_t b) {

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
 //   products in integers   exponents close to each other, as above
 //   products in FP64       exponents in the fixed-point range
 //   all in FP64            anything else: points too far apart for the range
-//                          (values below 2^-120 to 2^-1000), infinities, NaN,
+//                          (exponents above 120 to 1000), infinities, NaN,
 //                          entries below 2^-322
 //
 // Measured against the FP64 formula for every pair: 5003 x 20011 scattered

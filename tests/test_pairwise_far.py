@@ -1,7 +1,12 @@
 """FP64 pairwise products of points many correlation lengths apart: every value
 to its own size, wherever the kernel's exponent lies in the range of the
 fixed-point evaluation or beyond it (a sum over near and far pairs would hide
-the far ones). GPU against long double."""
+the far ones). Against long double: the evaluation compiled for the host, and
+the product on the GPU."""
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -89,3 +94,78 @@ def test_gaussian_operator_of_short_length(geometry, L):
         assert np.all(err <= 1e-12 * (absA @ np.abs(X).T).T)
     finally:
         kl.kl_destroy(h)
+
+
+HOST = r"""
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#include "fixed_gamma.cuh"
+#include <cstdio>
+using namespace kl;
+static const fx::Exp2Table TAB;
+typedef long double LD;
+// largest error of 2^-t, in units of 2^-53 of itself, for differences along one
+// direction and along the diagonal up to the largest exponent of the format
+template <int K> LD worst() {
+    LD w = 0;
+    const LD one = ldexpl(1, fx::Format<K>::kCoord);
+    for (int diag = 0; diag < 2; ++diag)
+        for (int i = 1; i <= 4000; ++i) {
+            const LD t = fx::Format<K>::kMaxArg * (LD)i / 4000;
+            const LD share = K == KL_KERNEL_EXP_SEP ? t / 3 : sqrtl((K == KL_KERNEL_GAUSS ? t : t * t) / 3);
+            const LD d = diag ? share : (K == KL_KERNEL_GAUSS ? sqrtl(t) : t);
+            const uint64_t u = (uint64_t)(d * one);
+            for (int back = 0; back < 2; ++back) {
+                const uint64_t x = fx::absdiff(back ? 0 : u, back ? u : 0), y = diag ? x : 0;
+                uint32_t n;
+                const uint64_t e = fx::exponent<K>(x, y, y);
+                const uint64_t E = fx::exp2_neg<fx::Format<K>::kArg>(e, TAB.v, n);
+                const LD c = (LD)u / one;
+                const LD q = K == KL_KERNEL_GAUSS ? c * c * (diag ? 3 : 1) : diag ? (K == KL_KERNEL_EXP_SEP ? 3 * c : c * sqrtl(3)) : c;
+                const LD r = fabsl(ldexpl((LD)E, -63) * exp2l(-(LD)n) / exp2l(-q) - 1) * ldexpl(1, 53);
+                if (!(r <= w)) w = r;
+            }
+        }
+    return w;
+}
+int main() {
+    printf("%.6Lg %.6Lg %.6Lg\n", worst<KL_KERNEL_GAUSS>(), worst<KL_KERNEL_EXP_SEP>(), worst<KL_KERNEL_EXP>());
+    return 0;
+}
+"""
+
+
+def test_host_full_range(tmp_path):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no g++")
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(HOST)
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2101_00629_gb300", "csrc")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I", csrc, "-o", str(exe), str(src)], check=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True).stdout.split()
+    # the exponential (below 0.5), and the exponent: one unit of 2^-55 (2^-53)
+    # per difference and one of the result, times ln 2; the reference's own
+    # exponent carries 64 bits of a number below 2^10
+    assert all(float(e) < 0.5 + 4 + 1 for e in out)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("S", [1, 32])
+@pytest.mark.parametrize("along", ["axis", "diagonal"])
+@pytest.mark.parametrize("kernel,most", [("gauss", 1000), ("exp_sep", 500), ("exp", 120), ("matern32", 120)])
+def test_every_exponent(kernel, most, along, S):
+    """One point and one compact group against targets at exponents (base 2)
+    from 0 to beyond the fixed-point range."""
+    T, L = 700, 0.5
+    t = np.linspace(0.0, 1.1 * most, T)
+    direction = np.array([1.0, 0.0, 0.0]) if along == "axis" else np.ones(3)
+    unit = direction.sum() if kernel == "exp_sep" else np.sqrt((direction ** 2).sum())
+    r = L * (np.sqrt(t * LN2) if kernel == "gauss" else t * LN2 / (np.sqrt(3) if kernel == "matern32" else 1)) / unit
+    tgt = 0.25 + direction[:, None] * r
+    src = np.full((3, S), 0.25)
+    src[1] += 0.003 * np.arange(S) / 32
+    src[2] += 0.002 * (np.arange(S) % 4)
+    X = np.random.default_rng(1).uniform(0.5, 1.0, (2, S))
+    _check(kernel, L, tgt, src, X)
