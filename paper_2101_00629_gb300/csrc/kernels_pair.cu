@@ -457,7 +457,10 @@ cudaError_t run_pair_reduce(const double* part, int splits, int64_t T, int k, do
 
 // Scale of a distance (Gauss: its square root is taken) in base-2 exponents,
 // to 64 bits: a log2(e) or sqrt(a log2(e)).
+// 1 / L or 1 / L^2 beyond the FP64 range (L below 1e-154 for the Gaussian)
+// leaves no scale: infinite, so that every group takes the FP64 formula.
 FxScale fx_scale(int kind, double a) {
+    if (!std::isfinite(a)) return {0, 0, INFINITY};
     int e;
     const double f = std::frexp(a, &e);                           // a = f 2^e, f in [1/2, 1)
     const uint64_t m = uint64_t(std::ldexp(f, 53));               // exact

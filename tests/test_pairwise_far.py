@@ -96,6 +96,25 @@ def test_gaussian_operator_of_short_length(geometry, L):
         kl.kl_destroy(h)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("L", [1e-320, 1e-310, 1e-300, 1e-160, 1e-100, 1e100, 1e200, 1e300])
+@pytest.mark.parametrize("kernel", ["gauss", "exp_sep", "exp", "matern32"])
+def test_extreme_lengths(kernel, L):
+    """Lengths whose inverse (or its square) leaves the FP64 range: what the
+    FP64 formula gives, NaN at coincident points among it."""
+    x = np.array([0.0, 1e-310, 1e-160, 1e-20, 1.0, 1e30])
+    Y = np.zeros(6)
+    for t in range(6):  # one target at a time: a warp takes one path
+        Y[t] = _product(kernel, L, np.array([[x[t]], [0.0], [0.0]]), np.zeros((3, 1)), np.ones((1, 1)))[0, 0]
+    with np.errstate(all="ignore"):
+        inv = np.float64(1.0) / np.float64(L * L) if kernel == "gauss" else np.float64(1.0) / np.float64(L)
+        if kernel == "matern32":
+            inv = np.sqrt(3.0) / np.float64(L)
+        s = inv * (x * x if kernel == "gauss" else np.sqrt(x * x) if kernel != "exp_sep" else x)
+        ref = np.exp(-s) * (1 + s if kernel == "matern32" else 1)
+    np.testing.assert_allclose(Y, ref, rtol=1e-12, atol=1e-322)
+
+
 HOST = r"""
 #define __host__
 #define __device__
