@@ -258,6 +258,15 @@ __device__ inline void givens_r(dfl x, dfl z, dfl& c, dfl& s, dfl& r) {
     r = dfl(rq.hi * isc, rq.lo * isc);
 }
 
+// 2^-e with 2^(e-1) <= m < 2^e, for products of numbers of size m to stay in
+// FP32's exponent range (FP64's needs no scaling)
+__device__ inline double pow2_inverse(double) { return 1.0; }
+__device__ inline float pow2_inverse(float m) {
+    const int e = ((__float_as_int(m) >> 23) & 0xff) - 126;
+    return m > 1e-37f && e <= 126 ? __int_as_float((127 - e) << 23) : 1.f;
+}
+__device__ inline dfl pow2_inverse(dfl m) { return dfl(pow2_inverse(m.hi), 0.f); }
+
 // complex numbers over the working arithmetic R
 template <class R>
 struct cpx {
@@ -1071,26 +1080,40 @@ __global__ void __launch_bounds__(kEigThreads) nonsym_eig_kernel(const double* _
                     s_fail = 1;
                     action = 4;
                 } else {
-                    R sh, th;
+                    // the two shifts: the roots of (x - y1)(x - y2) = wa wb
+                    R y1, y2, wa, wb;
                     if (s_its > 0 && s_its % 10 == 0) {  // exceptional shift
                         const R ex = fabs(A[u + int64_t(u - 1) * ld]) + fabs(A[(u - 1) + int64_t(u - 2) * ld]);
-                        const R c = A[u + int64_t(u) * ld] + R(0.75) * ex;
-                        sh = R(2.0) * c;
-                        th = c * c + R(0.4375) * ex * ex;
+                        y1 = y2 = A[u + int64_t(u) * ld] + R(0.75) * ex;
+                        wa = R(-0.4375) * ex;
+                        wb = ex;
                     } else {
-                        const R a = A[(u - 1) + int64_t(u - 1) * ld], b = A[(u - 1) + int64_t(u) * ld];
-                        const R c = A[u + int64_t(u - 1) * ld], d = A[u + int64_t(u) * ld];
-                        sh = a + d;
-                        th = a * d - b * c;
+                        y1 = A[u + int64_t(u) * ld];
+                        y2 = A[(u - 1) + int64_t(u - 1) * ld];
+                        wa = A[u + int64_t(u - 1) * ld];
+                        wb = A[(u - 1) + int64_t(u) * ld];
                     }
                     s_its = s_its + 1;
-                    // first column of (H - s1)(H - s2) restricted to the window
-                    const R h11 = A[l + int64_t(l) * ld], h12 = A[l + int64_t(l + 1) * ld];
-                    const R h21 = A[(l + 1) + int64_t(l) * ld], h22 = A[(l + 1) + int64_t(l + 1) * ld];
+                    // First column of (H - s1)(H - s2) restricted to the
+                    // window, from differences (as in Martin, Peters and
+                    // Wilkinson's hqr): in a cluster of equal eigenvalues the
+                    // entries are ||H|| and their differences 1e-10 of it, so
+                    // that h11^2 - (s1 + s2) h11 + s1 s2 is all rounding and
+                    // the steps do not converge (matrices of order 12 to 96
+                    // with threefold eigenvalues 3e-10 apart: 60 to 696 steps
+                    // and up to 13 entries of 1e-10 ||H|| dropped, against 21
+                    // to 181 steps and none). The column's length is free:
+                    // scaled, its products stay in the exponent range.
+                    const R h12 = A[l + int64_t(l + 1) * ld], h21 = A[(l + 1) + int64_t(l) * ld];
                     const R h32 = A[(l + 2) + int64_t(l + 1) * ld];
-                    s_x[0] = h11 * h11 + h12 * h21 - sh * h11 + th;
-                    s_x[1] = h21 * (h11 + h22 - sh);
-                    s_x[2] = h21 * h32;
+                    const R d1 = A[l + int64_t(l) * ld] - y1, d2 = A[l + int64_t(l) * ld] - y2;
+                    const R d3 = d1 + (A[(l + 1) + int64_t(l + 1) * ld] - y2);
+                    const R top = fmax(fmax(fmax(fabs(d1), fabs(d2)), fmax(fabs(wa), fabs(wb))),
+                                       fmax(fmax(fabs(h12), fabs(h21)), fmax(fabs(h32), fabs(d3))));
+                    const R sc = pow2_inverse(top), sd1 = sc * d1, s21 = sc * h21;
+                    s_x[0] = sd1 * (sc * d2) - (sc * wa) * (sc * wb) + (sc * h12) * s21;
+                    s_x[1] = s21 * (sc * d3);
+                    s_x[2] = s21 * (sc * h32);
                 }
             }
             if (action == 1) {

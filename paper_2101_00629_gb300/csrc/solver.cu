@@ -213,15 +213,6 @@ int rayleigh_ritz(Ctx& c, const double* V, const double* AV, int nv, double* max
                                            c.w.ibuf, c.h->stream, c.nvec, kEigFP64), "nonsym_eig"));
             KL_TRY(sync_copy(c, &status, c.w.ibuf, sizeof(int)));
         }
-        if (arith == kEigFP64 && status == 1) {
-            // FP64 deflates at the rounding level; clusters of the operator's
-            // rounding (narrow kernels, many wanted pairs) can resist it for
-            // any number of iterations. Double-float deflates at 1e-13 ||H||;
-            // the restarts that follow are in FP64 again.
-            KL_TRY(ck(c, launch_nonsym_eig(c.w.H, nv, c.w.theta, c.w.thetai, c.w.S, c.w.Q, c.w.la_work,
-                                           c.w.ibuf, c.h->stream, c.nvec, kEigDF), "nonsym_eig"));
-            KL_TRY(sync_copy(c, &status, c.w.ibuf, sizeof(int)));
-        }
         c.schur_ok = status == 0;
         if (status == 2) status = 0;  // complex pairs: eigenvectors valid, Schur order not
     }
