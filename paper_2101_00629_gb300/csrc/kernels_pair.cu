@@ -81,12 +81,29 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
 // 57-bit numbers relative to the largest of the group, in two limbs of 28 and
 // 29 bits, and three 32 x 32 -> 64-bit multiply-adds per column sum the group
 // exactly (the product of the two low limbs lies below the last bit kept).
-// One FP64 FMA per column and group adds the group to the running sum. A term
-// is off by 2^-58 of the group's largest value times its largest entry; an
-// FP64 evaluation rounds a value exp(-t ln 2) by (1.5 + t) 2^-53 of itself. The
-// groups that take this path have values within a factor 2^5 (1.5 + t) of each
-// other, t the largest exponent, so that even a group whose largest entry
-// meets its smallest value is no less exact than in FP64.
+// One FP64 FMA per column and group adds the group to the running sum.
+//
+// The integer form is off by at most
+//     2^-58 G (W + (n / 2 + c + 1) M),  W = sum |x|,
+// in a group with values below G and n non-zero entries below M, c of them
+// rounded: truncation of the values (half a unit is added back to each), rounding
+// of the entries and of the sum, and the dropped product (half of its range is
+// added back). An FP64 evaluation may be off by 2^-53 (0.75 + 0.35 t) g |x| in a
+// term (rounding of the exponential and one rounding of its exponent t, 2^-54 t
+// ln 2) and by 2^-53 g |x| for each of the r additions that follow, of which half
+// is counted. A group takes the integer form where its bound is the smaller one
+// in every column. The sum over g v, v = (0.75 + r / 2) |x|, is at least V = sum v
+// times the value at the mean squared distance with the weights v (all kernels
+// are convex in it; the separable one in each direction), which mean and
+// variance of the positions give; 0.35 t g is at least that of the farthest
+// source:
+//     V g(mean) + 0.35 t_max W g(t_max) >= 2^-5 G (W + (n / 2 + c + 1) M).
+// Groups with entries of one size pass up to values of 2^-6 G, groups that a far
+// and late entry dominates hardly ever. On lines of 0.25 to 5.5 correlation
+// lengths with equal, normal, graded, single and dominating entries the form
+// then is as exact as FP64 or better wherever it is taken, rms and largest
+// error. A limit on the values alone let through ten times FP64's error (an
+// entry of 1 behind 31 below 1e-8: 25 against 2.4 units of 2^-53 of sum g |x|, rms).
 //
 // A group is a block of the sources' tensor grid (SrcGrid), as near a cube as
 // the grid's spacing allows: 32 consecutive points of the half cylinder's
@@ -102,13 +119,14 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
 //                          entries below 2^-322
 //
 // Measured against the FP64 formula for every pair: 5003 x 20011 scattered
-// points, Matern-3/2, 3 columns, 8.13 -> 0.84 ms; half-cylinder Galerkin
-// operator, Euclidean exponential, 8 columns, 1.5e8 pairs, 10.7 -> 1.59 ms, and
-// its degree-6 Gaussian collocation operator, 3.7e8 pairs, 20.3 -> 2.94 ms (with
-// groups of 32 consecutive points 2.18 and 5.1 ms: FP64 products, that pipe
-// 93 to 97 % busy). Bound by the integer pipes: 83 to 172 instructions per pair
-// and about seven per column, three of them 32 x 32 -> 64-bit multiply-adds of
-// four issue cycles. Two targets per thread were 5 to 20 % slower (registers).
+// points, Matern-3/2, 3 columns, 8.14 -> 0.86 ms; half-cylinder Galerkin
+// operator, Euclidean exponential, 8 columns, 1.5e8 pairs, 10.7 -> 1.74 ms, and
+// its degree-6 Gaussian collocation operator, 3.7e8 pairs, 20.3 -> 3.54 ms (with
+// every group on FP64 products that pipe is 93 to 97 % busy; deciding without
+// the entries took 0.84, 1.60 and 2.94 ms at the errors above). Bound by the
+// integer pipes: 83 to 172 instructions per pair and about seven per column,
+// three of them 32 x 32 -> 64-bit multiply-adds of four issue cycles. Two targets
+// per thread were 5 to 20 % slower (registers).
 // Sources as a tensor grid n[0] x n[1] x n[2] (index i0 + n0 (i1 + n1 i2)) cut
 // into blocks of 2^s[0] x 2^s[1] x 2^s[2] points, 32 or fewer.
 struct SrcGrid {
@@ -149,8 +167,10 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     __shared__ __align__(16) uint64_t s_c[ST][4];
     __shared__ __align__(16) int2 s_xl[ST][KB];
     __shared__ __align__(16) double s_xd[ST][KB];
-    __shared__ float s_box[NG][6];
+    __shared__ float s_box[NG][6], s_quick[NG];
+    __shared__ float4 s_mean[NG][KB], s_var[NG][KB];
     __shared__ int s_emax[NG][KB];
+    __shared__ int64_t s_mean_low[NG][KB];
     __shared__ int s_special[NG], s_count[NG], s_emin[NG];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < 1024; i += kTgt)
@@ -195,6 +215,8 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             float lo[3] = {float(x - rx) * sc.f, float(y - ry) * sc.f, float(z - rz) * sc.f}, hi[3];
             bool bad = !(isfinite(lo[0]) && isfinite(lo[1]) && isfinite(lo[2]));
             int emin = 2047;
+            const float rel[3] = {lo[0], lo[1], lo[2]};
+            float quick = 16384.0f;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 hi[q] = lo[q];
@@ -204,6 +226,21 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                     hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
                 }
             }
+            // positions in the box, 500 units to its largest half edge, and
+            // their squares (EXP_SEP: one by one) over 2048
+            const float half_edge = 0.5f * fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2]));
+            const float unit = half_edge * 0.002f, per_unit = half_edge > 0.0f ? 500.0f / half_edge : 0.0f;
+            float centre[3];
+            int at[3], sq[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                centre[q] = 0.5f * (lo[q] + hi[q]);
+                at[q] = __float2int_rn((rel[q] - centre[q]) * per_unit);
+                sq[q] = at[q] * at[q];
+            }
+            if (KIND != KL_KERNEL_EXP_SEP) sq[0] += sq[1] + sq[2];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) sq[q] = (sq[q] + 1024) >> 11;
 #pragma unroll
             for (int c = 0; c < KB; ++c) {
                 const double xv = (v && c < kc) ? X[sj + int64_t(c0 + c) * ldx] : 0.0;
@@ -222,14 +259,49 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 if (rs <= 57) xi = int64_t((m + (rs ? uint64_t(1) << (rs - 1) : 0)) >> rs);
                 if (xv < 0.0) xi = -xi;
                 const int32_t x1 = int32_t((xi + (1 << 27)) >> 28);
-                if (v) s_xl[j][c] = make_int2(x1, int32_t(xi - (int64_t(x1) << 28)));
-                if (lane == 0) s_emax[g][c] = emax;
+                // entries' sizes (2^26 at most), their sum, and mean and
+                // variance of the position with the weights of the rule above
+                const unsigned some = __ballot_sync(0xffffffffu, b != 0);
+                const int cut = __popc(__ballot_sync(0xffffffffu, rs > 3 && b != 0));
+                const unsigned size = unsigned(x1 < 0 ? -x1 : x1) >> 2;
+                const float sum = float(__reduce_add_sync(0xffffffffu, size));
+                // 4 v 2^-16, at most 65 * 2^10 (30 bits with the positions)
+                const int weight = int(size >> 16) * int(2 * __popc(some >> lane) + 1);
+                const float total = float(__reduce_add_sync(0xffffffffu, weight)), r = 1.0f / total;
+                const float y0 = float(__reduce_add_sync(0xffffffffu, weight * at[0])) * r;
+                const float y1 = float(__reduce_add_sync(0xffffffffu, weight * at[1])) * r;
+                const float y2 = float(__reduce_add_sync(0xffffffffu, weight * at[2])) * r;
+                const float q0 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[0])) * r;
+                const float d = 32.0f / (sum + float(__popc(some) + 2 * cut + 2) * 33554432.0f);
+                float4 mean = make_float4(fmaf(y0, unit, centre[0]), fmaf(y1, unit, centre[1]),
+                                          fmaf(y2, unit, centre[2]), 16384.0f * total * d);
+                float4 var = make_float4(0.0f, 0.0f, 0.0f, 0.35f * sum * d);
+                if (KIND == KL_KERNEL_EXP_SEP) {
+                    const float q1 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[1])) * r;
+                    const float q2 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[2])) * r;
+                    var.x = fmaxf(q0 - y0 * y0, 0.0f) * (unit * unit);
+                    var.y = fmaxf(q1 - y1 * y1, 0.0f) * (unit * unit);
+                    var.z = fmaxf(q2 - y2 * y2, 0.0f) * (unit * unit);
+                } else {
+                    var.x = fmaxf(q0 - (y0 * y0 + y1 * y1 + y2 * y2), 0.0f) * (unit * unit);
+                }
+                if (some == 0) mean = make_float4(0.0f, 0.0f, 0.0f, 0.0f), var = make_float4(0.0f, 0.0f, 0.0f, 1e30f);
+                else quick = fminf(quick, mean.w);
+                if (lane == 0) s_mean[g][c] = mean, s_var[g][c] = var;
+                const int32_t x0 = int32_t(xi - (int64_t(x1) << 28));
+                if (v) s_xl[j][c] = make_int2(x1, x0);
+                const int half = __reduce_add_sync(0xffffffffu, (x1 + x0) >> 3);
+                if (lane == 0) {
+                    s_emax[g][c] = emax;
+                    s_mean_low[g][c] = int64_t(half) * 4 + (1 << 27);
+                }
             }
             const bool any_bad = __any_sync(0xffffffffu, bad);
             if (lane == 0) {
                 s_special[g] = any_bad;
                 s_count[g] = __popc(have);
                 s_emin[g] = emin;
+                s_quick[g] = quick;
 #pragma unroll
                 for (int q = 0; q < 3; ++q) s_box[g][q] = lo[q], s_box[g][3 + q] = hi[q];
             }
@@ -254,7 +326,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 thi = sqrtf(thi);
             }
             const bool in_range = tfinite && !s_special[g] && thi < fx::Format<KIND>::kMaxArg;
-            const float most = 5.0f + log2f(1.5f + thi);
+            const float far = thi + 1e-9f;
             int gm = 0;
             if (KIND == KL_KERNEL_MATERN32) {
                 const float fh = 1.0f + 0.6931472f * thi;
@@ -267,7 +339,26 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             const int n0 = int(fminf(tlo, 1000.0f));
             // the group's scale 2^(emax - 56 - n0) is a normal number in every
             // column (far Gaussian groups: n0 reaches 999)
-            const bool narrow = thi - float(n0) < most && n0 <= s_emin[g] - 57;
+            bool narrow = thi - float(n0) < 14.0f && n0 <= s_emin[g] - 57;
+            const float farthest = ex2_approx(float(n0) - thi);
+            // the rule with the farthest value in place of the mean, then the
+            // rule itself
+            if (!__all_sync(0xffffffffu, in_range && narrow && s_quick[g] * farthest >= 1.0f)) {
+#pragma unroll
+                for (int c = 0; c < KB; ++c) {
+                    const float4 mean = s_mean[g][c], var = s_var[g][c];
+                    const float dx = p[0] - mean.x, dy = p[1] - mean.y, dz = p[2] - mean.z;
+                    float t, f = 1.0f;
+                    if (KIND == KL_KERNEL_EXP_SEP)
+                        t = sqrt_approx(fmaf(dx, dx, var.x)) + sqrt_approx(fmaf(dy, dy, var.y)) + sqrt_approx(fmaf(dz, dz, var.z));
+                    else
+                        t = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, var.x)));
+                    if (KIND == KL_KERNEL_EXP || KIND == KL_KERNEL_MATERN32) t = sqrt_approx(t);
+                    if (KIND == KL_KERNEL_MATERN32) f = 1.0f + 0.6931472f * t;
+                    t = fmaf(t, 1.0f + 1e-5f, 1e-3f);
+                    narrow = narrow && fmaf(mean.w * f, ex2_approx(float(n0) - t), var.w * (far * farthest)) >= 1.0f;
+                }
+            }
             if (__all_sync(0xffffffffu, in_range && narrow)) {
                 int64_t hi[KB], mid[KB];
 #pragma unroll
@@ -304,11 +395,16 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 }
 #pragma unroll
                 for (int c = 0; c < KB; ++c) {
-                    const int64_t sum = hi[c] + (mid[c] >> 28);
+                    const int64_t sum = hi[c] + ((mid[c] + s_mean_low[g][c]) >> 28);
                     const double f = __longlong_as_double((long long)(s_emax[g][c] - 56 - n0) << 52);
                     acc[c] = fma(double(sum), f, acc[c]);
                 }
             } else if (__all_sync(0xffffffffu, in_range)) {
+                // the group's own sum first, as in the integer form: one
+                // rounding at the size of the running sum, not 32
+                double sum[KB];
+#pragma unroll
+                for (int c = 0; c < KB; ++c) sum[c] = 0.0;
                 for (int j = j0; j < j1; ++j) {
                     const uint64_t t = fx::exponent<KIND>(fx::absdiff(ux, s_c[j][0]), fx::absdiff(uy, s_c[j][1]),
                                                           fx::absdiff(uz, s_c[j][2]));
@@ -317,8 +413,10 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                     double gv = fx::to_double(E, nt);
                     if (KIND == KL_KERNEL_MATERN32) gv *= double(fx::matern_factor(t)) * 2.7755575615628914e-17;  // 2^-55
 #pragma unroll
-                    for (int c = 0; c < KB; ++c) acc[c] = fma(gv, s_xd[j][c], acc[c]);
+                    for (int c = 0; c < KB; ++c) sum[c] = fma(gv, s_xd[j][c], sum[c]);
                 }
+#pragma unroll
+                for (int c = 0; c < KB; ++c) acc[c] += sum[c];
             } else {
                 for (int j = j0; j < j1; ++j) {
                     const int64_t sj = int64_t(s_c[j][3]);

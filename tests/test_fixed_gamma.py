@@ -151,3 +151,50 @@ def test_pairwise_special_entries(bad):
     G = _gamma("exp", 0.7, P, Q)[0].astype(np.float64)
     ref = (X[:, None, :] * G[None]).sum(2)
     np.testing.assert_allclose(Y.cpu().numpy(), ref, rtol=1e-12, atol=1e-322)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("entries", ["far", "near", "graded", "descending", "single"])
+@pytest.mark.parametrize("length", [1.0, 3.0, 4.2, 5.5])
+@pytest.mark.parametrize("kernel", ["exp", "gauss", "matern32", "exp_sep"])
+def test_entries_of_unequal_size(kernel, length, entries):
+    """Groups of 32 sources on a line, the smallest values meeting the largest
+    entries: no more error than an FP64 evaluation may have. 64 groups, each the
+    only one that its column has entries in."""
+    import torch
+    import paper_2101_00629_gb300 as kl
+    n, groups, T = 32, 64, 32
+    rng = np.random.default_rng(11)
+    tgt, src = np.zeros((3, T)), np.zeros((3, groups * n))
+    tgt[0] = 1e-3 * rng.random(T)
+    pos = (np.arange(n) + rng.random((groups, n))) / n
+    src[0] = 0.002 + (length * pos if kernel != "gauss" else np.sqrt(length) * pos).ravel()
+    x = 1.0 + rng.random((groups, n))
+    tiny = 10.0 ** -rng.uniform(8, 17, (groups, n)) * rng.choice([-1.0, 1.0], (groups, n))
+    if entries == "far":
+        x[:, :-1] = tiny[:, :-1]
+    elif entries == "near":
+        x[:, 1:] = tiny[:, 1:]
+    elif entries == "graded":
+        x *= 10.0 ** -rng.uniform(0, 6, (groups, n))
+    elif entries == "descending":
+        x *= 10.0 ** (-8.0 * np.arange(n)[::-1] / n)
+    else:
+        x[:, :-1] = 0.0
+    X = np.zeros((groups, groups * n))
+    for g in range(groups):
+        X[g, g * n:(g + 1) * n] = x[g]
+    d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (tgt, src, X)]
+    Y = torch.empty(groups, T, dtype=torch.float64, device="cuda")
+    kl.kl_pairwise_noalloc(kernel, 1.0, 1.0, d[0], T, d[1], groups * n, d[2], groups * n, Y, T, groups,
+                           torch.cuda.current_stream())
+    Y = Y.cpu().numpy()
+    # FP64: the exponent a from a distance with roundings of 3.5 units of 2^-53 of
+    # itself, the exponential, the factor 1 + a and the product within 3 (5), and
+    # one rounding for each addition that follows
+    units = 5.0 if kernel == "matern32" else 3.0
+    for g in range(groups):
+        G, a = _gamma(kernel, 1.0, tgt.astype(np.longdouble), src[:, g * n:(g + 1) * n].astype(np.longdouble))
+        xl = x[g].astype(np.longdouble)
+        bound = ((units + 3.5 * a + np.arange(n)[::-1]) * G) @ np.abs(xl) * 2.0 ** -53
+        assert np.all(np.abs(Y[g] - G @ xl) <= bound)
