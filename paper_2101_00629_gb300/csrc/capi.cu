@@ -369,7 +369,8 @@ static int kron3_s(kl_solver* h, const double* const* Fd, const int* n_in, const
 
 // Y = Z^-1 X (both sweeps), L^-1 X (forward) or L^-T X (backward) through the
 // banded factors, one direction after the other; X and Y may be the same
-// block.
+// block (same leading dimension), but not overlap otherwise: the first
+// direction reads X and writes Y.
 static int line_solve3(kl_solver* h, bool fwd, bool bwd, const double* X, int64_t ldx, double* Y, int64_t ldy, int k,
                        const double* post = nullptr, const double* pre = nullptr) {
     int64_t a = 1, b = h->N;
@@ -655,7 +656,17 @@ int apply_operator(kl_solver* h, int which, int precision, const double* X, int6
 // Z^-1 (Kronecker LU solves, Sec. 3.2); with non-tensor NURBS weights
 // Z = diag(1 / W(x_i)) B diag(w), so Z^-1 = diag(1 / w) B^-1 diag(W(x_i)).
 int apply_zinv(kl_solver* h, const double* X, int64_t ldx, double* Y, int64_t ldy, int k) {
-    if (zinv_by_lines(h, k)) return line_solve3(h, true, true, X, ldx, Y, ldy, k, h->rat_invw, h->rat_Wc);
+    if (zinv_by_lines(h, k)) {
+        const bool apart = Y + (k - 1) * ldy + h->N <= X || X + (k - 1) * ldx + h->N <= Y;
+        if (!apart && !(X == Y && (ldx == ldy || k == 1))) {
+            cudaError_t e = launch_copy_block(X, ldx, h->ws[0], h->N, h->N, k, h->stream);
+            ++h->launches;
+            if (e != cudaSuccess) return cuda_fail(h, e, "copy");
+            X = h->ws[0];
+            ldx = h->N;
+        }
+        return line_solve3(h, true, true, X, ldx, Y, ldy, k, h->rat_invw, h->rat_Wc);
+    }
     return kron3(h, h->Zinv, h->N1, h->N1, X, ldx, Y, ldy, k, h->rat_invw, 0, 1, h->rat_Wc);
 }
 

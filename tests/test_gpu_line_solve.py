@@ -88,3 +88,27 @@ def test_standard_form_as_solves(geometry, p, elems, method):
             assert err <= 1e-12, (c, err)
     finally:
         kl.kl_destroy(h)
+
+
+@pytest.mark.parametrize("ldx,ldy,shift", [(0, 5, 0), (5, 0, 0), (0, 0, 7), (3, 0, -11)])
+@pytest.mark.parametrize("method", ["galerkin", "collocation"])
+def test_zinv_overlapping_blocks(method, ldx, ldy, shift):
+    """X and Y in one buffer with different leading dimensions or offsets."""
+    import torch
+    import paper_2101_00629_gb300 as kl
+    k = 64
+    h = kl.kl_create(kl.params(geometry="cube", degree=2, elems=(31, 17, 9), kernel="gauss", L=0.5, method=method),
+                     torch.cuda.current_stream())
+    try:
+        N, _, _ = kl.kl_dims(h)
+        X = torch.from_numpy(random_block(N, k, 3)).cuda()
+        Y = torch.empty_like(X)
+        kl.kl_apply_Zinv(h, X, N, Y, N, k)
+        buf = torch.zeros(k * (N + 16) + 64, dtype=torch.float64, device="cuda")
+        x = buf[32:].as_strided((k, N), (N + ldx, 1))
+        y = buf[32 + shift:].as_strided((k, N), (N + ldy, 1))
+        x.copy_(X)
+        kl.kl_apply_Zinv(h, x, N + ldx, y, N + ldy, k)
+        assert torch.equal(y, Y)
+    finally:
+        kl.kl_destroy(h)
