@@ -112,3 +112,37 @@ def test_zinv_overlapping_blocks(method, ldx, ldy, shift):
         assert torch.equal(y, Y)
     finally:
         kl.kl_destroy(h)
+
+
+@pytest.mark.parametrize("apply", ["Zinv", "Aprime"])
+@pytest.mark.parametrize("geometry,p,geo", [
+    ("projective_cube", 2, (0.5, 0.25, -0.2)),  # weights before and after the sweeps
+    ("projective_cube", 3, (-0.4, 0.3, 0.6)),
+    ("half_annulus", 2, (1.0, 2.0, 1.0)),       # Greville points of joined knots
+    ("half_annulus", 3, (1.0, 2.0, 1.0)),
+])
+def test_collocation_sweeps(geometry, p, geo, apply):
+    """Z^-1 and A' of a wide block (banded sweeps) against the same columns one
+    at a time (dense inverses)."""
+    import torch
+    import paper_2101_00629_gb300 as kl
+    k, elems = 64, (20, 14, 16)
+    h = kl.kl_create(kl.params(geometry=geometry, degree=p, elems=elems, kernel="gauss", L=0.8, method="collocation",
+                               precision="fp64", geo=geo), torch.cuda.current_stream())
+    try:
+        N, _, _ = kl.kl_dims(h)
+        call = kl.kl_apply_Zinv if apply == "Zinv" else kl.kl_apply_Aprime
+        X = torch.from_numpy(random_block(N, k, 13)).cuda()
+        Y, Y1 = torch.empty_like(X), torch.empty_like(X)
+        call(h, X, N, Y, N, k)
+        Z = [_one_d(Problem(geometry, p, elems, "gauss", 1.0, 0.8, geo=geo), "collocation", d) for d in range(3)]
+        cond = np.prod([np.linalg.norm(np.abs(np.linalg.inv(z)) @ np.abs(z), np.inf) for z in Z])
+        # two backward-stable solves by direction (at most 2 n units each), and
+        # for A' two pairwise products in other column blocks (1e-13)
+        tol = 8 * sum(z.shape[0] for z in Z) * cond * 2.0 ** -53 + (1e-13 * cond if apply == "Aprime" else 0.0)
+        for c in range(0, k, 21):
+            call(h, X[c], N, Y1[c], N, 1)
+            err = float((Y[c] - Y1[c]).abs().max() / Y1[c].abs().max())
+            assert err <= tol, (c, err, tol)
+    finally:
+        kl.kl_destroy(h)
