@@ -72,6 +72,32 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
     }
 }
 
+// Sources as a tensor grid n[0] x n[1] x n[2] (index i0 + n0 (i1 + n1 i2)) cut
+// into blocks of 2^s[0] x 2^s[1] x 2^s[2] points, 32 or fewer.
+struct SrcGrid {
+    int64_t n[3];
+    uint32_t nb[3];
+    int s[3];
+    __host__ __device__ int64_t groups() const { return int64_t(nb[0]) * nb[1] * nb[2]; }
+    // source of a lane of a group, -1 past the edge of the grid
+    __device__ int64_t source(uint32_t g, uint32_t lane) const {
+        const uint32_t g1 = g / nb[0], b0 = g - g1 * nb[0], b2 = g1 / nb[1], b1 = g1 - b2 * nb[1];
+        const int64_t i0 = (int64_t(b0) << s[0]) + (lane & ((1u << s[0]) - 1u));
+        const int64_t i1 = (int64_t(b1) << s[1]) + ((lane >> s[0]) & ((1u << s[1]) - 1u));
+        const int64_t i2 = (int64_t(b2) << s[2]) + ((lane >> (s[0] + s[1])) & ((1u << s[2]) - 1u));
+        const bool in = i0 < n[0] && i1 < n[1] && i2 < n[2] && (lane >> (s[0] + s[1] + s[2])) == 0;
+        return in ? i0 + n[0] * (i1 + n[1] * i2) : -1;
+    }
+};
+
+struct FxScale {
+    uint64_t m;  // scale of a distance in base-2 exponents: m 2^e
+    int e;
+    float f;     // the same, rounded
+};
+
+__device__ const fx::Exp2Table g_exp2 = fx::Exp2Table();
+
 // FP64 product with the kernel values in fixed point (fixed_gamma.cuh).
 //
 // Per pair the FP64 formula costs 20 to 40 FP64 operations for the value and
@@ -120,39 +146,15 @@ __global__ void __launch_bounds__(kTgt) pair_f64_kernel(
 //
 // Measured against the FP64 formula for every pair: 5003 x 20011 scattered
 // points, Matern-3/2, 3 columns, 8.14 -> 0.86 ms; half-cylinder Galerkin
-// operator, Euclidean exponential, 8 columns, 1.5e8 pairs, 10.7 -> 1.74 ms, and
-// its degree-6 Gaussian collocation operator, 3.7e8 pairs, 20.3 -> 3.54 ms (with
-// every group on FP64 products that pipe is 93 to 97 % busy; deciding without
-// the entries took 0.84, 1.60 and 2.94 ms at the errors above). Bound by the
-// integer pipes: 83 to 172 instructions per pair and about seven per column,
-// three of them 32 x 32 -> 64-bit multiply-adds of four issue cycles. Two targets
-// per thread were 5 to 20 % slower (registers).
-// Sources as a tensor grid n[0] x n[1] x n[2] (index i0 + n0 (i1 + n1 i2)) cut
-// into blocks of 2^s[0] x 2^s[1] x 2^s[2] points, 32 or fewer.
-struct SrcGrid {
-    int64_t n[3];
-    uint32_t nb[3];
-    int s[3];
-    __host__ __device__ int64_t groups() const { return int64_t(nb[0]) * nb[1] * nb[2]; }
-    // source of a lane of a group, -1 past the edge of the grid
-    __device__ int64_t source(uint32_t g, uint32_t lane) const {
-        const uint32_t g1 = g / nb[0], b0 = g - g1 * nb[0], b2 = g1 / nb[1], b1 = g1 - b2 * nb[1];
-        const int64_t i0 = (int64_t(b0) << s[0]) + (lane & ((1u << s[0]) - 1u));
-        const int64_t i1 = (int64_t(b1) << s[1]) + ((lane >> s[0]) & ((1u << s[1]) - 1u));
-        const int64_t i2 = (int64_t(b2) << s[2]) + ((lane >> (s[0] + s[1])) & ((1u << s[2]) - 1u));
-        const bool in = i0 < n[0] && i1 < n[1] && i2 < n[2] && (lane >> (s[0] + s[1] + s[2])) == 0;
-        return in ? i0 + n[0] * (i1 + n[1] * i2) : -1;
-    }
-};
-
-struct FxScale {
-    uint64_t m;  // scale of a distance in base-2 exponents: m 2^e
-    int e;
-    float f;     // the same, rounded
-};
-
-__device__ const fx::Exp2Table g_exp2 = fx::Exp2Table();
-
+// operator, Euclidean exponential, 8 columns, 1.5e8 pairs, 10.7 -> 1.72 ms, and
+// its degree-6 Gaussian collocation operator, 3.7e8 pairs, 20.3 -> 3.65 ms (every
+// group on FP64 products: 5 ms, that pipe 93 % busy; deciding without the
+// entries took 0.84, 1.60 and 2.94 ms at the errors above). Bound by the integer
+// pipes: 83 to 172 instructions per pair and about seven per column, three of
+// them 32 x 32 -> 64-bit multiply-adds of four issue cycles. Two targets per
+// thread were 5 to 20 % slower (registers). Half of a group's columns per warp
+// with 16 columns: 16^3 cube, Gaussian collocation, 8.9 -> 8.0 ms (7.6 ms without
+// the rule on the entries).
 template <int KIND, int KB>
 __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     const double* __restrict__ tx, const double* __restrict__ ty, const double* __restrict__ tz,
@@ -162,16 +164,20 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     chain_wait();
     constexpr int NG = KB > 8 ? 2 : 4;  // groups per stage
     constexpr int ST = 32 * NG;
+    // each warp stages a group's columns, two warps half of them each with two
+    // groups per stage
+    constexpr int PARTS = kTgt / 32 / NG, KP = KB / PARTS;
+    static_assert(PARTS * NG * 32 == kTgt && KP * PARTS == KB, "all warps stage");
     constexpr int Q = fx::Format<KIND>::kCoord, QA = fx::Format<KIND>::kArg;
     __shared__ __align__(16) uint64_t s_tab[2048];
     __shared__ __align__(16) uint64_t s_c[ST][4];
     __shared__ __align__(16) int2 s_xl[ST][KB];
     __shared__ __align__(16) double s_xd[ST][KB];
-    __shared__ float s_box[NG][6], s_quick[NG];
+    __shared__ float s_box[NG][6], s_quick[NG][PARTS];
     __shared__ float4 s_mean[NG][KB], s_var[NG][KB];
     __shared__ int s_emax[NG][KB];
     __shared__ int64_t s_mean_low[NG][KB];
-    __shared__ int s_special[NG], s_count[NG], s_emin[NG];
+    __shared__ int s_special[NG][PARTS], s_count[NG], s_emin[NG][PARTS];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < 1024; i += kTgt)
         reinterpret_cast<ulonglong2*>(s_tab)[i] = reinterpret_cast<const ulonglong2*>(g_exp2.v)[i];
@@ -195,10 +201,10 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
     for (int64_t base = s0; base < s1; base += NG) {
         const int ng = int(s1 - base < NG ? s1 - base : int64_t(NG));
         __syncthreads();
-        // one warp per group, one source per lane; a block of the grid that
+        // one warp per group (or half of its columns), one source per lane; a block of the grid that
         // reaches over its edge leaves lanes without a source, the others
         // move together
-        for (int g = warp; g < ng; g += kTgt / 32) {
+        if (const int g = warp / PARTS, share = warp % PARTS; g < ng) {
             const int64_t sj = sg.source(uint32_t(base) + g, lane);
             const unsigned have = __ballot_sync(0xffffffffu, sj >= 0);
             const bool v = sj >= 0;
@@ -206,7 +212,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             const int64_t sl = __shfl_sync(0xffffffffu, (long long)sj, __ffs(int(have)) - 1);
             const int64_t sv = v ? sj : sl;
             const double x = sx[sv], y = sy[sv], z = sz[sv];
-            if (v) {
+            if (v && share == 0) {
                 s_c[j][0] = fx::to_fixed<Q>(x, sc.m, sc.e);
                 s_c[j][1] = fx::to_fixed<Q>(y, sc.m, sc.e);
                 s_c[j][2] = fx::to_fixed<Q>(z, sc.m, sc.e);
@@ -226,23 +232,9 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                     hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
                 }
             }
-            // positions in the box, 500 units to its largest half edge, and
-            // their squares (EXP_SEP: one by one) over 2048
-            const float half_edge = 0.5f * fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2]));
-            const float unit = half_edge * 0.002f, per_unit = half_edge > 0.0f ? 500.0f / half_edge : 0.0f;
-            float centre[3];
-            int at[3], sq[3];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                centre[q] = 0.5f * (lo[q] + hi[q]);
-                at[q] = __float2int_rn((rel[q] - centre[q]) * per_unit);
-                sq[q] = at[q] * at[q];
-            }
-            if (KIND != KL_KERNEL_EXP_SEP) sq[0] += sq[1] + sq[2];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) sq[q] = (sq[q] + 1024) >> 11;
-#pragma unroll
-            for (int c = 0; c < KB; ++c) {
+            for (int cc = 0; cc < KP; ++cc) {
+                const int c = share * KP + cc;
                 const double xv = (v && c < kc) ? X[sj + int64_t(c0 + c) * ldx] : 0.0;
                 if (v) s_xd[j][c] = xv;
                 const uint64_t b = uint64_t(__double_as_longlong(xv)) & 0x7fffffffffffffffull;
@@ -259,35 +251,22 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 if (rs <= 57) xi = int64_t((m + (rs ? uint64_t(1) << (rs - 1) : 0)) >> rs);
                 if (xv < 0.0) xi = -xi;
                 const int32_t x1 = int32_t((xi + (1 << 27)) >> 28);
-                // entries' sizes (2^26 at most), their sum, and mean and
-                // variance of the position with the weights of the rule above
+                // entries' sizes (2^26 at most), their sum, and that of the
+                // weights v of the rule above; a mean position out of reach
+                // until it is formed below
                 const unsigned some = __ballot_sync(0xffffffffu, b != 0);
                 const int cut = __popc(__ballot_sync(0xffffffffu, rs > 3 && b != 0));
                 const unsigned size = unsigned(x1 < 0 ? -x1 : x1) >> 2;
                 const float sum = float(__reduce_add_sync(0xffffffffu, size));
                 // 4 v 2^-16, at most 65 * 2^10 (30 bits with the positions)
                 const int weight = int(size >> 16) * int(2 * __popc(some >> lane) + 1);
-                const float total = float(__reduce_add_sync(0xffffffffu, weight)), r = 1.0f / total;
-                const float y0 = float(__reduce_add_sync(0xffffffffu, weight * at[0])) * r;
-                const float y1 = float(__reduce_add_sync(0xffffffffu, weight * at[1])) * r;
-                const float y2 = float(__reduce_add_sync(0xffffffffu, weight * at[2])) * r;
-                const float q0 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[0])) * r;
+                const float total = float(__reduce_add_sync(0xffffffffu, weight));
                 const float d = 32.0f / (sum + float(__popc(some) + 2 * cut + 2) * 33554432.0f);
-                float4 mean = make_float4(fmaf(y0, unit, centre[0]), fmaf(y1, unit, centre[1]),
-                                          fmaf(y2, unit, centre[2]), 16384.0f * total * d);
-                float4 var = make_float4(0.0f, 0.0f, 0.0f, 0.35f * sum * d);
-                if (KIND == KL_KERNEL_EXP_SEP) {
-                    const float q1 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[1])) * r;
-                    const float q2 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[2])) * r;
-                    var.x = fmaxf(q0 - y0 * y0, 0.0f) * (unit * unit);
-                    var.y = fmaxf(q1 - y1 * y1, 0.0f) * (unit * unit);
-                    var.z = fmaxf(q2 - y2 * y2, 0.0f) * (unit * unit);
-                } else {
-                    var.x = fmaxf(q0 - (y0 * y0 + y1 * y1 + y2 * y2), 0.0f) * (unit * unit);
+                if (some) quick = fminf(quick, 16384.0f * total * d);
+                if (lane == 0) {
+                    s_mean[g][c] = make_float4(1e18f, 1e18f, 1e18f, some ? 16384.0f * total * d : 0.0f);
+                    s_var[g][c] = make_float4(0.0f, 0.0f, 0.0f, some ? 0.35f * sum * d : 1e30f);
                 }
-                if (some == 0) mean = make_float4(0.0f, 0.0f, 0.0f, 0.0f), var = make_float4(0.0f, 0.0f, 0.0f, 1e30f);
-                else quick = fminf(quick, mean.w);
-                if (lane == 0) s_mean[g][c] = mean, s_var[g][c] = var;
                 const int32_t x0 = int32_t(xi - (int64_t(x1) << 28));
                 if (v) s_xl[j][c] = make_int2(x1, x0);
                 const int half = __reduce_add_sync(0xffffffffu, (x1 + x0) >> 3);
@@ -296,14 +275,64 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                     s_mean_low[g][c] = int64_t(half) * 4 + (1 << 27);
                 }
             }
+            // the mean positions, where the quick test may fail: elsewhere the
+            // exponents of the box lie within its diameter of each other (not
+            // the Gaussian's, which grow with the distance)
+            const float diameter = (hi[0] - lo[0]) + (hi[1] - lo[1]) + (hi[2] - lo[2]);
+            if (KIND == KL_KERNEL_GAUSS || !(quick * ex2_approx(-1.01f * diameter - 1.1f) >= 1.0f)) {
+                // positions in the box, 500 units to its largest half edge, and
+                // their squares (EXP_SEP: one by one) over 2048
+                const float half_edge = 0.5f * fmaxf(hi[0] - lo[0], fmaxf(hi[1] - lo[1], hi[2] - lo[2]));
+                const float unit = half_edge * 0.002f, per_unit = half_edge > 0.0f ? 500.0f / half_edge : 0.0f;
+                float centre[3];
+                int at[3], sq[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    centre[q] = 0.5f * (lo[q] + hi[q]);
+                    at[q] = __float2int_rn((rel[q] - centre[q]) * per_unit);
+                    sq[q] = at[q] * at[q];
+                }
+                if (KIND != KL_KERNEL_EXP_SEP) sq[0] += sq[1] + sq[2];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) sq[q] = (sq[q] + 1024) >> 11;
+#pragma unroll
+                for (int cc = 0; cc < KP; ++cc) {
+                    const int c = share * KP + cc;
+                    const int x1 = v ? s_xl[j][c].x : 0;
+                    const unsigned some = __ballot_sync(0xffffffffu, v && s_xd[j][c] != 0.0);
+                    const int weight = int(unsigned(x1 < 0 ? -x1 : x1) >> 18) * int(2 * __popc(some >> lane) + 1);
+                    const float r = 1.0f / float(__reduce_add_sync(0xffffffffu, weight));
+                    const float y0 = float(__reduce_add_sync(0xffffffffu, weight * at[0])) * r;
+                    const float y1 = float(__reduce_add_sync(0xffffffffu, weight * at[1])) * r;
+                    const float y2 = float(__reduce_add_sync(0xffffffffu, weight * at[2])) * r;
+                    const float q0 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[0])) * r;
+                    float v0 = q0 - y0 * y0, v1 = 0.0f, v2 = 0.0f;
+                    if (KIND == KL_KERNEL_EXP_SEP) {
+                        v1 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[1])) * r - y1 * y1;
+                        v2 = 2048.0f * float(__reduce_add_sync(0xffffffffu, weight * sq[2])) * r - y2 * y2;
+                    } else {
+                        v0 -= y1 * y1 + y2 * y2;
+                    }
+                    if (lane == 0 && some) {
+                        s_mean[g][c].x = fmaf(y0, unit, centre[0]);
+                        s_mean[g][c].y = fmaf(y1, unit, centre[1]);
+                        s_mean[g][c].z = fmaf(y2, unit, centre[2]);
+                        s_var[g][c].x = fmaxf(v0, 0.0f) * (unit * unit);
+                        s_var[g][c].y = fmaxf(v1, 0.0f) * (unit * unit);
+                        s_var[g][c].z = fmaxf(v2, 0.0f) * (unit * unit);
+                    }
+                }
+            }
             const bool any_bad = __any_sync(0xffffffffu, bad);
             if (lane == 0) {
-                s_special[g] = any_bad;
-                s_count[g] = __popc(have);
-                s_emin[g] = emin;
-                s_quick[g] = quick;
+                s_special[g][share] = any_bad;
+                s_emin[g][share] = emin;
+                s_quick[g][share] = quick;
+                if (share == 0) {
+                    s_count[g] = __popc(have);
 #pragma unroll
-                for (int q = 0; q < 3; ++q) s_box[g][q] = lo[q], s_box[g][3 + q] = hi[q];
+                    for (int q = 0; q < 3; ++q) s_box[g][q] = lo[q], s_box[g][3 + q] = hi[q];
+                }
             }
         }
         __syncthreads();
@@ -325,7 +354,7 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
                 tlo = sqrtf(tlo);
                 thi = sqrtf(thi);
             }
-            const bool in_range = tfinite && !s_special[g] && thi < fx::Format<KIND>::kMaxArg;
+            const bool in_range = tfinite && !(s_special[g][0] | s_special[g][PARTS - 1]) && thi < fx::Format<KIND>::kMaxArg;
             const float far = thi + 1e-9f;
             int gm = 0;
             if (KIND == KL_KERNEL_MATERN32) {
@@ -339,11 +368,11 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
             const int n0 = int(fminf(tlo, 1000.0f));
             // the group's scale 2^(emax - 56 - n0) is a normal number in every
             // column (far Gaussian groups: n0 reaches 999)
-            bool narrow = thi - float(n0) < 14.0f && n0 <= s_emin[g] - 57;
+            bool narrow = thi - float(n0) < 14.0f && n0 <= min(s_emin[g][0], s_emin[g][PARTS - 1]) - 57;
             const float farthest = ex2_approx(float(n0) - thi);
             // the rule with the farthest value in place of the mean, then the
             // rule itself
-            if (!__all_sync(0xffffffffu, in_range && narrow && s_quick[g] * farthest >= 1.0f)) {
+            if (!__all_sync(0xffffffffu, in_range && narrow && fminf(s_quick[g][0], s_quick[g][PARTS - 1]) * farthest >= 1.0f)) {
 #pragma unroll
                 for (int c = 0; c < KB; ++c) {
                     const float4 mean = s_mean[g][c], var = s_var[g][c];
@@ -438,8 +467,9 @@ __global__ void __launch_bounds__(kTgt, KB > 8 ? 3 : 5) pair_fx_kernel(
 // 16-byte load) and its KB entries serve R pairs. Bound by instruction issue:
 // about 12 per value (two of them special-function), KB per product, and by
 // the FP64 additions of the tile sums. 2688 x 82368 points, Matern-3/2, whole
-// application: 5 columns 249 -> 205 us, 16 columns 455 -> 410 us against one
-// target per thread, scalar coordinate loads and 8 columns at least.
+// application: 5 columns 245 -> 205 us (198 us with dependent launches), 16
+// columns 455 -> 410 us against one target per thread, scalar coordinate loads
+// and 8 columns at least.
 template <int KIND, int KB, int R>
 __global__ void __launch_bounds__(kTgt) pair_f32_kernel(
     const float* __restrict__ tx, const float* __restrict__ ty, const float* __restrict__ tz,
