@@ -110,8 +110,10 @@ enum { KL_GALERKIN_IBQ = 0, KL_COLLOCATION = 1, KL_GALERKIN_STD = 2 };
  * the tolerance) are solved in FP32, and the returned pairs come from the
  * FP64 Rayleigh-Ritz refinement (`refine`).
  *   KL_FP64        kernel values and products to FP64 accuracy (CUDA cores:
- *                  64-bit fixed point where that is no less exact than FP64
- *                  arithmetic, FP64 elsewhere).
+ *                  64-bit fixed point where its error bound is below that
+ *                  of FP64 arithmetic for the entries given, FP64 elsewhere;
+ *                  the rounding of a vector can depend on the others of the
+ *                  same call).
  *   KL_FP32        FP32 kernel evaluation and FP32 products (CUDA cores).
  *   KL_MIXED_BF16  FP32 kernel tiles written to tensor memory and multiplied
  *                  on tcgen05 tensor cores as split (hi + lo) BF16 products
